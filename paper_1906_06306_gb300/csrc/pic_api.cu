@@ -1231,8 +1231,9 @@ pic_status pic_energies(pic_ctx* ctx, double* out, int nout) {
   for (int s = 0; s < ns; ++s) {
     PIC_CK(ctx, launch_kinetic(ctx->sp[s].u, ctx->sp[s].n, ctx->cap[s], (double)ctx->sp[s].m * c2,
                                ctx->d_acc + 2 + s, ctx->st));
-    PIC_CK(ctx, launch_rho(ctx->g, ctx->sp[s].cell, ctx->sp[s].off, ctx->sp[s].n, ctx->cap[s],
-                           (double)ctx->sp[s].q, ctx->d_rho, ctx->st));
+    PIC_CK(ctx, launch_rho(ctx->g, ctx->tile, ctx->d_tstart[s], ctx->sp[s].cell, ctx->sp[s].off,
+                           ctx->sorted_n[s], ctx->sp[s].n, ctx->cap[s], (double)ctx->sp[s].q,
+                           ctx->d_rho, ctx->st));
   }
   double* a = ctx->d_rho;
   double* b = ctx->d_rho2;

@@ -11,6 +11,15 @@ static unsigned blocks_for(long long n) {
   return (unsigned)(b < 1 ? 1 : b);
 }
 
+// Blocks of a reduction: every thread ends in a block sum of FP64 exchanges
+// (ten additions of the slow pipe), so a grid of 4 blocks per SM, each thread
+// with several terms, measures faster than one that fills the SMs (field
+// energy of a 1024^2 box 30.5 us with 16 blocks per SM).
+static unsigned blocks_for_sum(long long n) {
+  const unsigned b = blocks_for(n);
+  return b < 152u * 4u ? b : 152u * 4u;
+}
+
 __device__ __forceinline__ double block_sum(double v, double* sh) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -27,18 +36,81 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   return s;  // valid in thread 0
 }
 
+// Double-float arithmetic: a value as the unevaluated sum h + l of two floats,
+// |l| <= ulp(h)/2 (Dekker 1971; the error-free sum is Knuth's, the error-free
+// product the fused multiply-add's).  The GPU's FP64 pipe issues one operation
+// for some thirty FP32 ones, so the diagnostics form their terms, 46 to 48
+// bits of them, in FP32 pairs and keep FP64 for the sums over many terms.
+struct DF {
+  float h, l;
+};
+__device__ __forceinline__ DF two_sum(float a, float b) {
+  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+__device__ __forceinline__ DF fast_two_sum(float a, float b) {  // |a| >= |b| or a == 0
+  const float s = __fadd_rn(a, b);
+  return {s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+__device__ __forceinline__ DF square(float a) {
+  const float p = __fmul_rn(a, a);
+  return {p, __fmaf_rn(a, a, -p)};
+}
+__device__ __forceinline__ void add_to(DF& s, DF x) {  // s.l collects what s.h rounds off
+  const DF t = two_sum(s.h, x.h);
+  s.h = t.h;
+  s.l = __fadd_rn(s.l, __fadd_rn(t.l, x.l));
+}
+// approximations with a relative error below 2^-22 for normal arguments
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// Range of magnitudes whose squares a double-float holds with all its bits.
+constexpr float kDfMin = 9.094947e-13f;   // 2^-40
+constexpr float kDfMax = 1.1529215e18f;   // 2^60
+__device__ __forceinline__ bool df_range(float m) { return m >= kDfMin && m <= kDfMax; }
+
+constexpr int kDfTerms = 16;  // terms summed in double-float before the FP64 sum takes them
+
+// Sums of E^2 and B^2.  Squares are exact in double-float; every 16 points the
+// sums go on in FP64 (1024^2 box: 40 us with FP64 products, 22 us).
 __global__ void k_field_energy(const float* __restrict__ F, long long P, double* acc) {
   __shared__ double sh[32];
   double se = 0.0, sb = 0.0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P;
-       i += (long long)gridDim.x * blockDim.x) {
+  DF e = {0.f, 0.f}, b = {0.f, 0.f};
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  int terms = 0;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P; i += stride) {
+    float v[6];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const double e = F[(EX + a) * P + i], b = F[(BX + a) * P + i];
-      se += e * e;
-      sb += b * b;
+    for (int a = 0; a < 6; ++a) v[a] = F[(EX + a) * P + i];
+    bool ok = true;
+#pragma unroll
+    for (int a = 0; a < 6; ++a) ok &= v[a] == 0.f || df_range(fabsf(v[a]));
+    if (ok) {
+#pragma unroll
+      for (int a = 0; a < 6; ++a) add_to(a < 3 ? e : b, square(v[a]));
+    } else {
+#pragma unroll
+      for (int a = 0; a < 6; ++a) (a < 3 ? se : sb) += (double)v[a] * v[a];
+    }
+    if (++terms == kDfTerms) {
+      terms = 0;
+      se += (double)e.h + e.l;
+      sb += (double)b.h + b.l;
+      e = b = {0.f, 0.f};
     }
   }
+  se += (double)e.h + e.l;
+  sb += (double)b.h + b.l;
   se = block_sum(se, sh);
   sb = block_sum(sb, sh);
   if (threadIdx.x == 0) {
@@ -47,49 +119,243 @@ __global__ void k_field_energy(const float* __restrict__ F, long long P, double*
   }
 }
 
-// m c^2 (gamma - 1) with gamma - 1 = u^2 / (gamma + 1)
-__global__ void k_kinetic(const float* __restrict__ u, long long n, long long ld, double mc2,
-                          double* acc) {
+// gamma - 1 = u^2 / (gamma + 1) in double-float, for max |u_a| in df_range:
+// the squares and their sum without error, gamma and the quotient by one
+// Newton correction each of their FP32 values (relative error below 2^-44).
+__device__ __forceinline__ DF gamma_minus_1(float a, float b, float c) {
+  const DF pa = square(a), pb = square(b), pc = square(c);
+  const DF s1 = two_sum(pa.h, pb.h), s2 = two_sum(s1.h, pc.h);
+  const DF u2 = fast_two_sum(s2.h, ((pa.l + pb.l) + pc.l) + (s1.l + s2.l));
+  const DF x = two_sum(1.0f, u2.h);
+  const float y = rsqrt_approx(x.h), g0 = __fmul_rn(x.h, y);
+  const float g1 = __fmul_rn(__fadd_rn(__fmaf_rn(-g0, g0, x.h), __fadd_rn(x.l, u2.l)), 0.5f * y);
+  const DF d = two_sum(g0, 1.0f);
+  const float r = rcp_approx(d.h), t = __fmul_rn(u2.h, r);
+  const float rem = __fmaf_rn(-t, __fadd_rn(d.l, g1), __fadd_rn(__fmaf_rn(-t, d.h, u2.h), u2.l));
+  return {t, __fmul_rn(rem, r)};
+}
+
+// Sum of m c^2 (gamma - 1).  With square root and quotient in FP64 the FP64
+// pipe bounded it, 769 us for 16.8 M particles; with terms in double-float and
+// 16 of them to an FP64 addition it takes 60 us, bound by FP32 issue (the
+// reads alone would take 30 us).
+__global__ void __launch_bounds__(256) k_kinetic(const float* __restrict__ u, long long n,
+                                                 long long ld, double mc2, double* acc) {
   __shared__ double sh[32];
   double s = 0.0;
-  for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n;
-       p += (long long)gridDim.x * blockDim.x) {
-    const double a = u[p], b = u[ld + p], c = u[2 * ld + p];
-    const double u2 = a * a + b * b + c * c;
-    s += u2 / (sqrt(1.0 + u2) + 1.0);
+  DF sum = {0.f, 0.f};
+  int terms = 0;
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  constexpr int U = 4;  // rounds whose loads are issued together
+  for (long long base = blockIdx.x * (long long)blockDim.x + threadIdx.x; base < n;
+       base += U * stride) {
+    float v[U][3];
+#pragma unroll
+    for (int r = 0; r < U; ++r) {
+      const long long p = base + r * stride;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) v[r][a] = p < n ? u[a * ld + p] : 0.f;
+    }
+#pragma unroll
+    for (int r = 0; r < U; ++r) {
+      const float m = fmaxf(fabsf(v[r][0]), fmaxf(fabsf(v[r][1]), fabsf(v[r][2])));
+      const bool at_rest = v[r][0] == 0.f && v[r][1] == 0.f && v[r][2] == 0.f;
+      const bool nan = v[r][0] != v[r][0] || v[r][1] != v[r][1] || v[r][2] != v[r][2];
+      if (df_range(m) && !nan) {
+        add_to(sum, gamma_minus_1(v[r][0], v[r][1], v[r][2]));
+      } else if (!at_rest) {
+        const double a = v[r][0], b = v[r][1], c = v[r][2];
+        const double u2 = a * a + b * b + c * c;
+        s += u2 / (sqrt(1.0 + u2) + 1.0);
+      }
+    }
+    terms += U;
+    if (terms == kDfTerms) {
+      terms = 0;
+      s += (double)sum.h + sum.l;
+      sum = {0.f, 0.f};
+    }
   }
+  s += (double)sum.h + sum.l;
   s = block_sum(s, sh);
   if (threadIdx.x == 0) atomicAdd(acc, mc2 * s);
 }
 
 // charge q with weights (1 - w, w) per gridded axis onto the 2^D nodes
 template <int D>
+__device__ __forceinline__ void rho_particle(const GridDev& g, int c, const float* o, double q,
+                                             double* rho) {
+  int ijk[3];
+  ijk[0] = c % g.n[0];
+  const int r = c / g.n[0];
+  ijk[1] = r % g.n[1];
+  ijk[2] = r / g.n[1];
+  double w[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int d = 0; d < D; ++d) w[d] = o[d];
+#pragma unroll
+  for (int corner = 0; corner < (1 << D); ++corner) {
+    double wt = q;
+    int id[3] = {ijk[0], ijk[1], ijk[2]};
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      const int up = (corner >> d) & 1;
+      wt *= up ? w[d] : 1.0 - w[d];
+      id[d] = up ? wrap1(id[d] + 1, g.n[d]) : id[d];
+    }
+    atomicAdd(&rho[id[0] + (long long)g.n[0] * (id[1] + (long long)g.n[1] * id[2])], wt);
+  }
+}
+
+template <int D>
 __global__ void k_rho(const GridDev g, const int* __restrict__ cell, const float* __restrict__ off,
-                      long long n, long long ld, double q, double* rho) {
-  for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n;
+                      long long first, long long n, long long ld, double q, double* rho) {
+  for (long long p = first + blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n;
        p += (long long)gridDim.x * blockDim.x) {
     const int c = cell[p];
     if (c < 0 || (long long)c >= g.plane) continue;
-    int ijk[3];
-    ijk[0] = c % g.n[0];
-    const int r = c / g.n[0];
-    ijk[1] = r % g.n[1];
-    ijk[2] = r / g.n[1];
-    double w[3] = {0.0, 0.0, 0.0};
+    float o[3] = {0.f, 0.f, 0.f};
 #pragma unroll
-    for (int d = 0; d < D; ++d) w[d] = off[d * ld + p];
+    for (int d = 0; d < D; ++d) o[d] = off[d * ld + p];
+    rho_particle<D>(g, c, o, q, rho);
+  }
+}
+
+// The same charge for particles grouped by tile (1D and 2D), by fixed-point
+// sums in shared memory.  A block takes its share of a tile's bucket and sums,
+// for each cell of the tile's window, the particle count and the moments
+// sum w_x, sum w_y, sum w_x w_y in units of 2^-48; the four corner weights of
+// every particle are differences of these (w_x - w_x w_y, ...), so a node's
+// charge is one integer sum over its four cells, rounded once to FP64.
+// Each moment goes as three 16-bit limbs into 32-bit words with native
+// integer atomics (64-bit shared atomics are a compare-and-swap loop), so
+// kRhoBatch = 2^15 particles can neither overflow a word nor the 64-bit
+// sums.  An offset has 24 significant bits: a moment is short of its exact
+// value by less than 2^-47, below the rounding of an FP64 sum of 16 charges.
+// Particles outside the window, or whose offsets are not in [0, 1), take the
+// FP64 atomics of k_rho, and so does the unsorted tail.  The global atomics
+// bounded that kernel (one FP64 atomic per L2 slice and clock: 4 a particle,
+// 338 us for 16.8 M in 2D); here a block issues one per window node, and the
+// kernel takes 95 us, bound by the 10 shared atomics a particle.  Four rounds
+// of loads go out together (135 us with one).
+constexpr int kRhoBatch = 1 << 15;
+
+template <int D>
+__host__ __device__ constexpr int rho_words() {
+  return 1 + 3 * ((1 << D) - 1);
+}
+
+// A float w in [0, 1) is m 2^(e - 150), m < 2^24.
+__device__ __forceinline__ unsigned mantissa(float w) {
+  return (__float_as_uint(w) & 0x7fffffu) | 0x800000u;
+}
+__device__ __forceinline__ int exponent(float w) { return (int)((__float_as_uint(w) >> 23) & 255u); }
+__device__ __forceinline__ unsigned long long shifted(unsigned long long m, int sh) {
+  return sh >= 0 ? m << sh : (sh > -64 ? m >> -sh : 0ULL);
+}
+
+template <int D>
+__global__ void __launch_bounds__(256, 6) k_rho_tiles(const GridDev g, const TileDev t, int splits,
+                                                   FastDiv div0, const int* __restrict__ tstart,
+                                                   const int* __restrict__ cell,
+                                                   const float* __restrict__ off, long long ld,
+                                                   double q, double* rho) {
+  extern __shared__ unsigned sw[];
+  constexpr int NW = rho_words<D>();
+  const int tile = blockIdx.x / splits, split = blockIdx.x - tile * splits;
+  const int w0[2] = {(tile % t.nt[0]) * t.T[0] - t.H, D == 2 ? (tile / t.nt[0]) * t.T[1] - t.H : 0};
+  const int W0 = t.W[0], W1 = D == 2 ? t.W[1] : 1, wc = W0 * W1;
+  const bool near = W0 <= g.n[0] && (D < 2 || W1 <= g.n[1]);
+  const long long lo = tstart[tile * t.nsub], len = tstart[(tile + 1) * t.nsub] - lo;
+  const long long a = lo + len * split / splits, b = lo + len * (split + 1) / splits;
+  for (long long first = a; first < b; first += kRhoBatch) {
+    const long long last = first + kRhoBatch < b ? first + kRhoBatch : b;
+    for (int w = threadIdx.x; w < NW * wc; w += blockDim.x) sw[w] = 0u;
+    __syncthreads();
+    constexpr int U = 4;  // rounds whose loads are issued together
+    for (long long base = first + threadIdx.x; base < last; base += U * blockDim.x) {
+      int cu[U];
+      float ou[U][2];
 #pragma unroll
-    for (int corner = 0; corner < (1 << D); ++corner) {
-      double wt = q;
-      int id[3] = {ijk[0], ijk[1], ijk[2]};
-#pragma unroll
-      for (int d = 0; d < D; ++d) {
-        const int o = (corner >> d) & 1;
-        wt *= o ? w[d] : 1.0 - w[d];
-        id[d] = o ? wrap1(id[d] + 1, g.n[d]) : id[d];
+      for (int r = 0; r < U; ++r) {
+        const long long p = base + r * blockDim.x;
+        cu[r] = p < last ? cell[p] : -1;
+        ou[r][0] = p < last ? off[p] : 0.f;
+        ou[r][1] = D == 2 && p < last ? off[ld + p] : 0.f;
       }
-      atomicAdd(&rho[id[0] + (long long)g.n[0] * (id[1] + (long long)g.n[1] * id[2])], wt);
+#pragma unroll
+      for (int r = 0; r < U; ++r) {
+        const int c = cu[r];
+        const float* o = ou[r];
+        if (c < 0 || (long long)c >= g.plane) continue;
+        const int j = D == 2 ? fdiv(c, div0) : 0, i = c - j * g.n[0];
+        int l0 = i - w0[0], l1 = D == 2 ? j - w0[1] : 0;
+        if (near) {  // at most one period away
+          l0 = wrap1(l0, g.n[0]);
+          if (D == 2) l1 = wrap1(l1, g.n[1]);
+        } else {
+          l0 = wrapi(l0, g.n[0]);
+          if (D == 2) l1 = wrapi(l1, g.n[1]);
+        }
+        bool in = l0 < W0 - 1 && o[0] >= 0.f && o[0] < 1.f;
+        if (D == 2) in &= l1 < W1 - 1 && o[1] >= 0.f && o[1] < 1.f;
+        if (in) {
+          unsigned* s = sw + l0 + W0 * l1;
+          unsigned long long m[3];
+          const unsigned mx = mantissa(o[0]);
+          const int ex = exponent(o[0]) - 102;  // units of 2^-48
+          m[0] = shifted(mx, ex);
+          if (D == 2) {
+            const unsigned my = mantissa(o[1]);
+            const int ey = exponent(o[1]) - 150;
+            m[1] = shifted(my, ey + 48);
+            m[2] = shifted((unsigned long long)mx * my, ex + ey);
+          }
+          atomicAdd(s, 1u);
+  #pragma unroll
+          for (int k = 0; k < (1 << D) - 1; ++k) {
+            atomicAdd(s + (1 + 3 * k) * wc, (unsigned)m[k] & 0xffffu);
+            atomicAdd(s + (2 + 3 * k) * wc, (unsigned)m[k] >> 16);
+            atomicAdd(s + (3 + 3 * k) * wc, (unsigned)(m[k] >> 32));
+          }
+        } else {
+          rho_particle<D>(g, c, o, q, rho);
+        }
+      }
     }
+    __syncthreads();
+    for (int w = threadIdx.x; w < wc; w += blockDim.x) {
+      const int lx = w % W0, ly = w / W0;
+      // moments of cell v: {count 2^48, w_x, w_y, w_x w_y}
+      auto cell_sums = [&](int v, long long* m) {
+        m[0] = (long long)sw[v] << 48;
+#pragma unroll
+        for (int k = 0; k < (1 << D) - 1; ++k)
+          m[1 + k] = (long long)sw[v + (1 + 3 * k) * wc] +
+                     ((long long)sw[v + (2 + 3 * k) * wc] << 16) +
+                     ((long long)sw[v + (3 + 3 * k) * wc] << 32);
+      };
+      long long sum = 0, m[4];
+      cell_sums(w, m);
+      sum += D == 1 ? m[0] - m[1] : m[0] - m[1] - m[2] + m[3];
+      if (lx > 0) {
+        cell_sums(w - 1, m);
+        sum += D == 1 ? m[1] : m[1] - m[3];
+      }
+      if (D == 2 && ly > 0) {
+        cell_sums(w - W0, m);
+        sum += m[2] - m[3];
+        if (lx > 0) {
+          cell_sums(w - W0 - 1, m);
+          sum += m[3];
+        }
+      }
+      if (sum != 0) {
+        const int i = wrapi(w0[0] + lx, g.n[0]), j = D == 2 ? wrapi(w0[1] + ly, g.n[1]) : 0;
+        atomicAdd(&rho[i + (long long)g.n[0] * j], q * ((double)sum * 0x1p-48));
+      }
+    }
+    __syncthreads();
   }
 }
 
@@ -132,33 +398,61 @@ __global__ void k_gauss(const GridDev g, const float* __restrict__ F, const doub
 }
 
 cudaError_t launch_field_energy(const GridDev& g, const float* F, double* acc, cudaStream_t st) {
-  k_field_energy<<<blocks_for(g.plane), 256, 0, st>>>(F, g.plane, acc);
+  k_field_energy<<<blocks_for_sum(g.plane), 256, 0, st>>>(F, g.plane, acc);
   return cudaGetLastError();
 }
 
 cudaError_t launch_kinetic(const float* u, long long n, long long ld, double mc2, double* acc,
                            cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  k_kinetic<<<blocks_for(n), 256, 0, st>>>(u, n, ld, mc2, acc);
+  k_kinetic<<<blocks_for_sum(n), 256, 0, st>>>(u, n, ld, mc2, acc);
   return cudaGetLastError();
 }
 
-cudaError_t launch_rho(const GridDev& g, const int* cell, const float* off, long long n,
-                       long long ld, double q, double* rho, cudaStream_t st) {
-  if (n == 0) return cudaSuccess;
-  const unsigned nb = blocks_for(n);
+static cudaError_t launch_rho_global(const GridDev& g, const int* cell, const float* off,
+                                     long long first, long long n, long long ld, double q,
+                                     double* rho, cudaStream_t st) {
+  if (n <= first) return cudaSuccess;
+  const unsigned nb = blocks_for(n - first);
   switch (g.dim) {
-    case 1: k_rho<1><<<nb, 256, 0, st>>>(g, cell, off, n, ld, q, rho); break;
-    case 2: k_rho<2><<<nb, 256, 0, st>>>(g, cell, off, n, ld, q, rho); break;
-    case 3: k_rho<3><<<nb, 256, 0, st>>>(g, cell, off, n, ld, q, rho); break;
+    case 1: k_rho<1><<<nb, 256, 0, st>>>(g, cell, off, first, n, ld, q, rho); break;
+    case 2: k_rho<2><<<nb, 256, 0, st>>>(g, cell, off, first, n, ld, q, rho); break;
+    case 3: k_rho<3><<<nb, 256, 0, st>>>(g, cell, off, first, n, ld, q, rho); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
 }
 
+// The tile kernel for the grouped particles of 1D and 2D boxes (about 8192 of
+// them to a block, so that zeroing and folding a window stay small), and the
+// global one for what follows them.  3D takes the global kernel: eight moments
+// of an 8x8x4 tile's window would take 134 KB of shared memory.
+cudaError_t launch_rho(const GridDev& g, const TileDev& t, const int* tstart, const int* cell,
+                       const float* off, long long sorted, long long n, long long ld, double q,
+                       double* rho, cudaStream_t st) {
+  if (n == 0) return cudaSuccess;
+  const size_t smem = sizeof(unsigned) * (g.dim == 1 ? rho_words<1>() : rho_words<2>()) * (size_t)t.wcells;
+  if (g.dim == 3 || sorted == 0 || smem > 200 * 1024)
+    return launch_rho_global(g, cell, off, 0, n, ld, q, rho, st);
+  const void* k = g.dim == 1 ? (const void*)k_rho_tiles<1> : (const void*)k_rho_tiles<2>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  if (e != cudaSuccess) return e;
+  long long splits = (sorted / t.ntiles + 8191) / 8192;
+  splits = splits < 1 ? 1 : splits > 1024 ? 1024 : splits;
+  const unsigned nb = (unsigned)(t.ntiles * splits);
+  const FastDiv d0 = make_fastdiv(g.n[0]);
+  if (g.dim == 1)
+    k_rho_tiles<1><<<nb, 256, smem, st>>>(g, t, (int)splits, d0, tstart, cell, off, ld, q, rho);
+  else
+    k_rho_tiles<2><<<nb, 256, smem, st>>>(g, t, (int)splits, d0, tstart, cell, off, ld, q, rho);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  return launch_rho_global(g, cell, off, sorted, n, ld, q, rho, st);
+}
+
 cudaError_t launch_gauss(const GridDev& g, const float* F, const double* rho, int i_lo, int i_hi,
                          unsigned long long* acc_max, double* acc_sq, cudaStream_t st) {
-  const unsigned nb = blocks_for(g.plane);
+  const unsigned nb = blocks_for_sum(g.plane);
   switch (g.dim) {
     case 1: k_gauss<1><<<nb, 256, 0, st>>>(g, F, rho, i_lo, i_hi, acc_max, acc_sq); break;
     case 2: k_gauss<2><<<nb, 256, 0, st>>>(g, F, rho, i_lo, i_hi, acc_max, acc_sq); break;

@@ -268,8 +268,11 @@ cudaError_t launch_unpermute(const int* perm, const float* in, float* out, long 
 cudaError_t launch_field_energy(const GridDev& g, const float* F, double* acc, cudaStream_t st);
 cudaError_t launch_kinetic(const float* u, long long n, long long ld, double mc2, double* acc,
                            cudaStream_t st);
-cudaError_t launch_rho(const GridDev& g, const int* cell, const float* off, long long n,
-                       long long ld, double q, double* rho, cudaStream_t st);
+// charge on the nodes of particles [0, n), of which the first `sorted` are
+// grouped by the buckets tstart of the tiling t (adds to rho)
+cudaError_t launch_rho(const GridDev& g, const TileDev& t, const int* tstart, const int* cell,
+                       const float* off, long long sorted, long long n, long long ld, double q,
+                       double* rho, cudaStream_t st);
 // over the nodes with i_lo <= i < i_hi: acc_max (as the bit pattern of a
 // non-negative double), acc_sq += sum res^2
 // one warp whose bounded barrier wait runs out (sets ST_TIMEOUT)
