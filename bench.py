@@ -110,7 +110,7 @@ def kernel_source_hash() -> str:
 def launches_per_step(sim, shock=False):
     """Kernels of a graph-replayed pic_step on `sim`'s tuning, per step and per
     sort cycle: per step the first B half step, the tile particle kernel, one
-    fused launch per filter pass, the deferred-particle kernel in 3D or with
+    launch per filter pass (less those of fused_away), the deferred-particle kernel in 3D or with
     the wall, and the second B half step with the E update (two launches; on a
     periodic FDTD2 lattice of at most 4096 points one launch that also takes
     the next step's first B half step, whose launch then opens only each
@@ -124,6 +124,15 @@ def launches_per_step(sim, shock=False):
     step = (1 if small else 3) + 1 + tun["filter_passes"] + (1 if sim.dim == 3 or shock else 0)
     sort = (3 if B.pic_sort_bins(sim.ctx) <= 4096 else 5) * sim.nspecies + (1 if small else 0)
     return step, sort
+
+
+def fused_away(sim):
+    """Filter passes of a step that need no launch of their own: up to four
+    passes share one in 1D and 2D, two in 3D, in an even number of launches
+    (one for a single pass)."""
+    passes = sim.tuning()["filter_passes"]
+    most = 2 if sim.dim == 3 else 4
+    return 0 if passes < 2 else passes - 2 * -(-passes // (2 * most))
 
 
 def profiled_traffic(workload, full_size, nparticles):
@@ -882,6 +891,7 @@ def run_ours(args):
     step_alg = step_bytes(pl, avg_n, tun["filter_passes"], tun["sort_every"])
     nsorts = -(-args.steps // tun["sort_every"])  # at most one sort per cadence in the loop
     per_step, per_sort = launches_per_step(sim, shock)
+    per_step -= fused_away(sim)
     launches = args.steps * per_step + nsorts * per_sort
     if shock:  # per step: 3 wall-field passes, the injection, and the tail kernel on
         # every step that does not start with a sort
@@ -1012,6 +1022,7 @@ def run_batched(args):
     launches = 0
     for sm in sims:
         per_step, per_sort = launches_per_step(sm)
+        per_step -= fused_away(sm)
         launches += args.steps * per_step + -(-args.steps // sm.tuning()["sort_every"]) * per_sort
     line = {
         "metric": METRIC, "value": value, "unit": "particle-steps/s", "n_gpus": world,
@@ -1123,9 +1134,9 @@ def run_adjoint(args):
     avg_adj = adj_ms * 1e-3 / max(adj_n, 1)
     # kernels behind the library's timed calls: a push is the tile kernel (2D,
     # periodic: no deferred-particle kernel), an adjoint step (tile pass) the B
-    # rebuild, 2 adjoint B half steps, the adjoint E update, one per filter
-    # pass, a bucket check per species, the tile pass and the deferred pass
-    passes = sim.tuning()["filter_passes"]
+    # rebuild, 2 adjoint B half steps, the adjoint E update, the filter's
+    # launches, a bucket check per species, the tile pass and the deferred pass
+    passes = sim.tuning()["filter_passes"] - fused_away(sim)
     launches = (kt["push"][1] + kt["b_half"][1] + kt["e_update"][1] + kt["filter"][1] +
                 kt["sort"][1] + (6 + passes + sim.nspecies) * kt["adjoint"][1])
     # per adjoint step: particle state read (4 + 8 + 12 B) and gradients read and

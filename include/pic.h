@@ -121,7 +121,8 @@ typedef struct {
                                at most 4096 points: with the second B half step,
                                and inside a multi-step pic_step call with the
                                next step's first B half step, in one launch) */
-#define PIC_KERNEL_FILTER 3 /* one Binomial2 pass */
+#define PIC_KERNEL_FILTER 3 /* one launch of Binomial2 passes (up to four in
+                               1D and 2D, two in 3D) */
 #define PIC_KERNEL_SORT 4   /* tile sort: count + scan + scatter + copy back */
 #define PIC_KERNEL_BOUNDARY 5 /* wall fields and injection (pic_set_shock) */
 #define PIC_KERNEL_ADJOINT 6  /* pic_adjoint_step */

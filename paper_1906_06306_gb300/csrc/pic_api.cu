@@ -628,10 +628,12 @@ pic_status do_filter(pic_ctx* ctx, int passes) {
   if (!ctx->d_jtmp) PIC_CK(ctx, dalloc(&ctx->d_jtmp, 3 * (size_t)ctx->g.plane));
   float* a = J;
   float* b = ctx->d_jtmp;
-  for (int p = 0; p < passes; ++p) {
+  for (int n = filter_launches(ctx->g.dim, passes); n > 0; --n) {
+    const int k = (passes + n - 1) / n;  // of the passes left, this launch's share
     const cudaError_t e = timed(
-        ctx, PIC_KERNEL_FILTER, [&]() { return launch_filter_pass_f32(ctx->g, a, b, 3, ctx->st, ctx->d_status); });
+        ctx, PIC_KERNEL_FILTER, [&]() { return launch_filter(ctx->g, a, b, 3, k, ctx->st, ctx->d_status); });
     if (e != cudaSuccess) return cuda_fail(ctx, "binomial filter", e);
+    passes -= k;
     float* t = a;
     a = b;
     b = t;
@@ -956,8 +958,11 @@ pic_status pic_adjoint_step(pic_ctx* ctx, const float* fwd_fields, const pic_adj
     float* J = adj_fields + JX * P;
     float* a = J;
     float* b = ctx->d_jtmp;
-    for (int p = 0; p < ctx->tun.filter_passes && r == cudaSuccess; ++p) {  // Jf = F^p J
-      r = launch_filter_pass_f32(ctx->g, a, b, 3, ctx->st, ctx->d_status);
+    int left = ctx->tun.filter_passes;  // Jf = F^p J
+    for (int n = filter_launches(ctx->g.dim, left); n > 0 && r == cudaSuccess; --n) {
+      const int k = (left + n - 1) / n;
+      r = launch_filter(ctx->g, a, b, 3, k, ctx->st, ctx->d_status);
+      left -= k;
       float* t = a;
       a = b;
       b = t;

@@ -72,11 +72,6 @@ constexpr bool kFoldGlobal = D == 3 && (PIC_X3PAIR != 0 || PIC_FOLD_GLOBAL_3D !=
 #ifndef PIC_TMA_WINDOW
 #define PIC_TMA_WINDOW 1
 #endif
-// The 2D/3D filter passes stage their rows by bulk copies (cp.async.bulk)
-// where the rows allow it and a status word can report a wait that ran out.
-#ifndef PIC_BULK_FILTER
-#define PIC_BULK_FILTER 1
-#endif
 // Resident blocks per SM the 1D/2D adjoint tile pass is compiled for (4: 64
 // registers without spills, 4 x 45 KB of shared memory for a 16x16-tile
 // window; measured 0.38 -> 0.27 ms per adjoint step of the 256^2 box against 2
@@ -217,19 +212,17 @@ cudaError_t launch_e_update(const GridDev& g, float* F, cudaStream_t st);
 constexpr long long kSmallFieldCells = 4096;
 bool fields_small_ok(const GridDev& g);
 cudaError_t launch_fields_small(const GridDev& g, float* F, cudaStream_t st, int chain = 0);
-// one Binomial2 sub-pass along gridded axis `axis` over ncomp consecutive planes,
-// src -> dst (a full pass is one sub-pass per gridded axis, x first)
-cudaError_t launch_filter_f32(const GridDev& g, const float* src, float* dst, int ncomp, int axis,
-                              cudaStream_t st);
+// `passes` Binomial2 passes (up to 4, in 3D up to 2) over ncomp consecutive
+// planes, src -> dst (src != dst), in one launch, and how many such launches
+// p passes take.  With a status word, 3D rows are staged by bulk copies whose
+// bounded waits report there; without one (nullptr) by per-thread copies.
+cudaError_t launch_filter(const GridDev& g, const float* src, float* dst, int ncomp, int passes,
+                          cudaStream_t st, int* status);
+int filter_launches(int dim, int passes);
+// one Binomial2 sub-pass along gridded axis `axis` over ncomp consecutive
+// planes, src -> dst (a full pass is one sub-pass per gridded axis, x first)
 cudaError_t launch_filter_f64(const GridDev& g, const double* src, double* dst, int ncomp,
                               int axis, cudaStream_t st);
-// one full Binomial2 pass (every gridded axis, x first) over ncomp consecutive
-// planes, src -> dst, the sub-passes fused through shared memory; with a
-// status word (2D/3D, aligned rows) the rows are staged by bulk copies whose
-// bounded waits report there, without one (nullptr) by per-thread copies
-cudaError_t launch_filter_pass_f32(const GridDev& g, const float* src, float* dst, int ncomp,
-                                   cudaStream_t st, int* status);
-
 struct SortParams {
   GridDev g;
   TileDev t;

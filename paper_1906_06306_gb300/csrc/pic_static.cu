@@ -77,9 +77,11 @@ extern "C" pic_status pic_filter_current_static(const pic_grid* grid, float* J, 
   // between J and the static scratch
   float* a = J;
   float* b = scratch;
-  for (int p = 0; p < passes; ++p) {
-    e = pic::launch_filter_pass_f32(g, a, b, 3, st, nullptr);
+  for (int n = pic::filter_launches(g.dim, passes); n > 0; --n) {
+    const int k = (passes + n - 1) / n;
+    e = pic::launch_filter(g, a, b, 3, k, st, nullptr);
     if (e != cudaSuccess) return fail(PIC_ERR_CUDA, cudaGetErrorString(e));
+    passes -= k;
     float* t = a;
     a = b;
     b = t;
