@@ -110,8 +110,8 @@ def kernel_source_hash() -> str:
 def launches_per_step(sim, shock=False):
     """Kernels of a graph-replayed pic_step on `sim`'s tuning, per step and per
     sort cycle: per step the first B half step, the tile particle kernel, one
-    launch per filter pass (less those of fused_away), the deferred-particle kernel in 3D or with
-    the wall, and the second B half step with the E update (two launches; on a
+    launch per filter pass (fused_away: those that share one), the
+    deferred-particle kernel in 3D or with the wall, and the second B half step with the E update (two launches; on a
     periodic FDTD2 lattice of at most 4096 points one launch that also takes
     the next step's first B half step, whose launch then opens only each
     cycle); per sort and species the count, the scan (three kernels past 4096
