@@ -25,6 +25,7 @@ namespace pic {
 // Adjoint of E' = E + c curl- B2 - Jf:  Bbar += c curl+ Ebar,  Jbar = -Ebar.
 template <int D>
 __global__ void k_adj_e(float* __restrict__ A, const GridDev g, float c) {
+  grid_dependency();
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
   const long long P = g.plane;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -62,6 +63,7 @@ __global__ void k_adj_e(float* __restrict__ A, const GridDev g, float c) {
 // Reads only B planes and writes only E planes, so the points are independent.
 template <int D>
 __global__ void k_adj_b(float* __restrict__ A, const GridDev g, float h) {
+  grid_dependency();
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
   const long long P = g.plane;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -381,6 +383,7 @@ __device__ __forceinline__ void cell_ijk(const AdjParams& P, int cell, int* b) {
 // particles listed by k_adj_tiles.
 template <int D>
 __global__ void __launch_bounds__(256) k_adj_particles(const AdjParams P, int deferred) {
+  grid_dependency();
   const GlobAcc F{const_cast<float*>(P.F1), P.g.plane, P.g.n[0], P.g.n[1], P.g.n[2]};
   const GlobAcc Ab{P.A, P.g.plane, P.g.n[0], P.g.n[1], P.g.n[2]};
   const float c = P.g.c;
@@ -474,6 +477,7 @@ __device__ __forceinline__ void adj_share(const AdjParams& P, const AdjSpecies& 
 template <int D>
 __global__ void __launch_bounds__(256, D == 3 ? 2 : PIC_ADJ_MIN_BLOCKS)
     k_adj_tiles(const AdjParams P) {
+  grid_dependency();
   extern __shared__ __align__(16) float sm[];
   __shared__ unsigned wmax[8];  // per warp of the block (256 threads)
   const AdjBlock B = adj_block<D>(P);
@@ -602,9 +606,9 @@ __global__ void __launch_bounds__(256, D == 3 ? 2 : PIC_ADJ_MIN_BLOCKS)
 cudaError_t launch_adj_e(const GridDev& g, float* A, cudaStream_t st) {
   const RowLaunch L = row_launch(g);
   switch (g.dim) {
-    case 1: k_adj_e<1><<<L.grid, L.threads, 0, st>>>(A, g, g.c); break;
-    case 2: k_adj_e<2><<<L.grid, L.threads, 0, st>>>(A, g, g.c); break;
-    case 3: k_adj_e<3><<<L.grid, L.threads, 0, st>>>(A, g, g.c); break;
+    case 1: launch_kernel(g.pdl, k_adj_e<1>, L.grid, L.threads, 0, st, A, g, g.c); break;
+    case 2: launch_kernel(g.pdl, k_adj_e<2>, L.grid, L.threads, 0, st, A, g, g.c); break;
+    case 3: launch_kernel(g.pdl, k_adj_e<3>, L.grid, L.threads, 0, st, A, g, g.c); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -614,9 +618,9 @@ cudaError_t launch_adj_b_half(const GridDev& g, float* A, cudaStream_t st) {
   const RowLaunch L = row_launch(g);
   const float h = 0.5f * g.c;
   switch (g.dim) {
-    case 1: k_adj_b<1><<<L.grid, L.threads, 0, st>>>(A, g, h); break;
-    case 2: k_adj_b<2><<<L.grid, L.threads, 0, st>>>(A, g, h); break;
-    case 3: k_adj_b<3><<<L.grid, L.threads, 0, st>>>(A, g, h); break;
+    case 1: launch_kernel(g.pdl, k_adj_b<1>, L.grid, L.threads, 0, st, A, g, h); break;
+    case 2: launch_kernel(g.pdl, k_adj_b<2>, L.grid, L.threads, 0, st, A, g, h); break;
+    case 3: launch_kernel(g.pdl, k_adj_b<3>, L.grid, L.threads, 0, st, A, g, h); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -650,9 +654,9 @@ cudaError_t launch_adj_particles(const AdjParams& P, cudaStream_t st) {
     const long long blocks = (long long)P.t.ntiles * P.splits;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
     switch (D) {
-      case 1: k_adj_tiles<1><<<(unsigned)blocks, 256, smem, st>>>(P); break;
-      case 2: k_adj_tiles<2><<<(unsigned)blocks, 256, smem, st>>>(P); break;
-      case 3: k_adj_tiles<3><<<(unsigned)blocks, 256, smem, st>>>(P); break;
+      case 1: launch_kernel(P.g.pdl, k_adj_tiles<1>, (unsigned)blocks, 256, smem, st, P); break;
+      case 2: launch_kernel(P.g.pdl, k_adj_tiles<2>, (unsigned)blocks, 256, smem, st, P); break;
+      case 3: launch_kernel(P.g.pdl, k_adj_tiles<3>, (unsigned)blocks, 256, smem, st, P); break;
       default: return cudaErrorInvalidValue;
     }
     e = cudaGetLastError();
@@ -664,9 +668,9 @@ cudaError_t launch_adj_particles(const AdjParams& P, cudaStream_t st) {
   if (nb > 152LL * 32) nb = 152LL * 32;
   const int deferred = tiled ? 1 : 0;
   switch (D) {
-    case 1: k_adj_particles<1><<<(unsigned)nb, 256, 0, st>>>(P, deferred); break;
-    case 2: k_adj_particles<2><<<(unsigned)nb, 256, 0, st>>>(P, deferred); break;
-    case 3: k_adj_particles<3><<<(unsigned)nb, 256, 0, st>>>(P, deferred); break;
+    case 1: launch_kernel(P.g.pdl, k_adj_particles<1>, (unsigned)nb, 256, 0, st, P, deferred); break;
+    case 2: launch_kernel(P.g.pdl, k_adj_particles<2>, (unsigned)nb, 256, 0, st, P, deferred); break;
+    case 3: launch_kernel(P.g.pdl, k_adj_particles<3>, (unsigned)nb, 256, 0, st, P, deferred); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

@@ -461,7 +461,7 @@ cudaError_t sort_species(pic_ctx* ctx, int s, bool copy_back, int32_t* perm) {
   r = launch_tile_count(P, ctx->sp[s].cell, n, ctx->d_count, ctx->st);
   if (r != cudaSuccess) return r;
   r = launch_tile_scan(ctx->d_count, bins, ctx->d_tstart[s], ctx->d_cursor, ctx->d_count + bins,
-                       ctx->st);
+                       ctx->st, ctx->g.pdl);
   if (r != cudaSuccess) return r;
   if (n == 0) return cudaSuccess;
   int* cell_out = (int*)ctx->d_sortbuf + sortbuf_offset(ctx, s);
@@ -622,7 +622,10 @@ pic_status step_capture(pic_ctx* ctx) {
   return PIC_OK;
 }
 
-pic_status do_filter(pic_ctx* ctx, int passes) {
+// `out` (where given) receives the planes that the result is in; without it
+// the result goes to the J planes.
+pic_status do_filter(pic_ctx* ctx, int passes, float** out = nullptr) {
+  if (out) *out = ctx->F + JX * ctx->g.plane;
   if (passes <= 0) return PIC_OK;
   float* J = ctx->F + JX * ctx->g.plane;
   if (!ctx->d_jtmp) PIC_CK(ctx, dalloc(&ctx->d_jtmp, 3 * (size_t)ctx->g.plane));
@@ -638,7 +641,9 @@ pic_status do_filter(pic_ctx* ctx, int passes) {
     a = b;
     b = t;
   }
-  if (a != J)
+  if (out)
+    *out = a;
+  else if (a != J)
     PIC_CK(ctx, cudaMemcpyAsync(J, a, sizeof(float) * 3 * ctx->g.plane, cudaMemcpyDeviceToDevice,
                                 ctx->st));
   return PIC_OK;
@@ -707,6 +712,7 @@ pic_status pic_init(pic_ctx** out, const pic_grid* grid, const pic_species* spec
   ctx->g.plane = ncell;
   ctx->g.c = c;
   ctx->g.order = 2;
+  ctx->g.pdl = 1;
   // defaults: tiles of 64 cells in 1D, 16^2 in 2D, 8x8x4 in 3D; sort every 10 steps
   // (3 in 3D, where a 2-cell halo is all the shared memory affords)
   ctx->tun.tile[0] = grid->dim == 1 ? 64 : grid->dim == 2 ? 16 : 8;
@@ -933,7 +939,7 @@ pic_status pic_adjoint_step(pic_ctx* ctx, const float* fwd_fields, const pic_adj
       int* t = ctx->d_adj_tstart + (long long)s * (nb + 1);
       PIC_CK(ctx, cudaMemcpyAsync(t, sp[s].tstart, sizeof(int) * (nb + 1),
                                   cudaMemcpyDeviceToDevice, ctx->st));
-      PIC_CK(ctx, launch_check_buckets(t, nb, ctx->sp[s].n, ctx->d_status, ctx->st));
+      PIC_CK(ctx, launch_check_buckets(t, nb, ctx->sp[s].n, ctx->d_status, ctx->st, ctx->g.pdl));
       S.tstart = t;
     }
     S.dlist = ctx->d_dlist + o;
@@ -1028,7 +1034,7 @@ pic_status pic_sort_assume(pic_ctx* ctx, const int32_t* const* tstart) {
     // a tile kernel must never read a slot outside [0, n): starts that are
     // not a partition are replaced by one bucket (correct, through the stray
     // path) and reported by pic_check
-    PIC_CK(ctx, launch_check_buckets(ctx->d_tstart[s], nb, n, ctx->d_status, ctx->st));
+    PIC_CK(ctx, launch_check_buckets(ctx->d_tstart[s], nb, n, ctx->d_status, ctx->st, ctx->g.pdl));
     ctx->sorted_n[s] = n;
   }
   ctx->snapshot_valid = false;
@@ -1100,7 +1106,8 @@ pic_status pic_field_update(pic_ctx* ctx, int which) {
   if (which == PIC_FIELD_B_HALF)
     e = timed(ctx, PIC_KERNEL_BHALF, [&]() { return launch_b_half(ctx->g, ctx->F, 0, ctx->st); });
   else if (which == PIC_FIELD_E)
-    e = timed(ctx, PIC_KERNEL_EUPD, [&]() { return launch_e_update(ctx->g, ctx->F, ctx->st); });
+    e = timed(ctx, PIC_KERNEL_EUPD,
+              [&]() { return launch_e_update(ctx->g, ctx->F, ctx->F + JX * ctx->g.plane, ctx->st); });
   else
     return set_err(ctx, PIC_ERR_ARG, "which must be PIC_FIELD_B_HALF or PIC_FIELD_E");
   if (e != cudaSuccess) return cuda_fail(ctx, "field update", e);
@@ -1126,22 +1133,23 @@ cudaError_t wall_fields(pic_ctx* ctx) {
 // periodic lattices only) the next step's first B half step too.
 pic_status step_fields(pic_ctx* ctx, bool chain = false) {
   cudaError_t e;
+  float* J = nullptr;
   if (!ctx->shock && fields_small_ok(ctx->g)) {
     // small periodic lattice: the filter (on J) first, then the second B
     // half step and the E update in one launch (the B half step touches B
     // only, the filter J only: the order between them does not matter)
-    const pic_status s = do_filter(ctx, ctx->tun.filter_passes);
+    const pic_status s = do_filter(ctx, ctx->tun.filter_passes, &J);
     if (s != PIC_OK) return s;
     e = timed(ctx, PIC_KERNEL_EUPD,
-              [&]() { return launch_fields_small(ctx->g, ctx->F, ctx->st, chain ? 1 : 0); });
+              [&]() { return launch_fields_small(ctx->g, ctx->F, J, ctx->st, chain ? 1 : 0); });
     if (e != cudaSuccess) return cuda_fail(ctx, "B half step and E update", e);
   } else {
     e = timed(ctx, PIC_KERNEL_BHALF, [&]() { return launch_b_half(ctx->g, ctx->F, 0, ctx->st); });
     if (e == cudaSuccess) e = wall_fields(ctx);
     if (e != cudaSuccess) return cuda_fail(ctx, "B half step", e);
-    const pic_status s = do_filter(ctx, ctx->tun.filter_passes);
+    const pic_status s = do_filter(ctx, ctx->tun.filter_passes, &J);
     if (s != PIC_OK) return s;
-    e = timed(ctx, PIC_KERNEL_EUPD, [&]() { return launch_e_update(ctx->g, ctx->F, ctx->st); });
+    e = timed(ctx, PIC_KERNEL_EUPD, [&]() { return launch_e_update(ctx->g, ctx->F, J, ctx->st); });
     if (e == cudaSuccess) e = wall_fields(ctx);
     if (e != cudaSuccess) return cuda_fail(ctx, "E update", e);
   }
@@ -1680,10 +1688,12 @@ pic_status batch_capture(pic_batch* b) {
     c->st = b->branches[i % b->branches.size()];
     c->timing = false;
     c->ensemble = true;
+    c->g.pdl = 0;  // blocks set up early would hold room that other boxes' blocks could use
     c->capturing = true;
     st = pic_step(c, b->cycle);
     c->capturing = false;
     c->ensemble = false;
+    c->g.pdl = 1;
     c->st = saved_st[i];
     c->timing = saved_timing[i];
     c->steps = saved_steps[i];  // the captured steps have not run yet

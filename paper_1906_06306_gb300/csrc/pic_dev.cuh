@@ -104,12 +104,22 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned b
       : "memory");
 }
 
+// Programmatic dependent launch: wait until every kernel before this one on the
+// stream is complete and its writes are visible, then let the next one be set
+// up.  In this order: once a kernel runs, all but the one before it are
+// complete.
+__device__ __forceinline__ void grid_dependency() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 struct GridDev {
   int dim;
   int n[3];          // cells per axis (1 for non-gridded axes)
   long long plane;   // n0*n1*n2
   float c;           // Courant number
   int order;         // spatial order of the field solver: 2 (FDTD2) or 4 (FDTD4)
+  int pdl;           // launches may overlap the kernel before them (launch_kernel)
 };
 
 struct TileDev {

@@ -46,6 +46,7 @@ __device__ __forceinline__ void b_half_point(float* __restrict__ F, const GridDe
 
 template <int D>
 __global__ void k_b_half(float* __restrict__ F, const GridDev g, float hc, int zero_j) {
+  grid_dependency();
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n0) return;
@@ -54,8 +55,8 @@ __global__ void k_b_half(float* __restrict__ F, const GridDev g, float hc, int z
 
 // E += c curl- B - J (backward differences: E sits half a cell below B).
 template <int D>
-__device__ __forceinline__ void e_update_point(float* __restrict__ F, const GridDev& g, int i,
-                                               int j, int k, float c) {
+__device__ __forceinline__ void e_update_point(float* __restrict__ F, const float* J,
+                                               const GridDev& g, int i, int j, int k, float c) {
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
   const long long P = g.plane;
   const long long idx = (long long)i + (long long)n0 * (j + (long long)n1 * k);
@@ -77,45 +78,66 @@ __device__ __forceinline__ void e_update_point(float* __restrict__ F, const Grid
     cx -= by - By[idx - sz];
     cy += bx - Bx[idx - sz];
   }
-  F[EX * P + idx] = fmaf(c, cx, F[EX * P + idx]) - F[JX * P + idx];
-  F[EY * P + idx] = fmaf(c, cy, F[EY * P + idx]) - F[JY * P + idx];
-  F[EZ * P + idx] = fmaf(c, cz, F[EZ * P + idx]) - F[JZ * P + idx];
+  const float jx = J[idx], jy = J[P + idx], jz = J[2 * P + idx];
+  F[EX * P + idx] = fmaf(c, cx, F[EX * P + idx]) - jx;
+  F[EY * P + idx] = fmaf(c, cy, F[EY * P + idx]) - jy;
+  F[EZ * P + idx] = fmaf(c, cz, F[EZ * P + idx]) - jz;
+  if (J != F + JX * P) {  // the filter left it in its buffer
+    F[JX * P + idx] = jx;
+    F[JY * P + idx] = jy;
+    F[JZ * P + idx] = jz;
+  }
 }
 
 template <int D>
-__global__ void k_e_update(float* __restrict__ F, const GridDev g, float c) {
+__global__ void k_e_update(float* __restrict__ F, const float* J, const GridDev g, float c) {
+  grid_dependency();
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n0) return;
-  FOR_ROWS(j, k) { e_update_point<D>(F, g, i, j, k, c); }
+  FOR_ROWS(j, k) { e_update_point<D>(F, J, g, i, j, k, c); }
 }
 
-// The second B half step and the E update of a small lattice by one block:
-// every point's B half step, a block barrier (which orders the block's
-// global-memory writes before its later reads), every point's E update; the
+// The second B half step and the E update of a small lattice by one block, in
+// shared memory: the planes are read once, every point's B half step, a
+// block barrier, every point's E update, and the planes are written once; the
 // operations of k_b_half and k_e_update point by point, so the same bits.  One
-// launch instead of two where launch latency, not bandwidth, bounds the step.
-// With `chain` set, after another barrier, the next step's first B half step
-// (which clears J for its deposit) as well: one launch instead of three.
+// launch instead of two where launch and memory latency, not bandwidth, bound
+// the step.  With `chain` set, after another barrier, the next step's first B
+// half step (which clears J for its deposit) as well: one launch instead of
+// three.  512 points: 7.0 us with the loads of a plane one after the other, 3.4
+// with all nine in flight (5.6 us with every phase in global memory).
 template <int D>
-__global__ void __launch_bounds__(1024) k_fields_small(float* __restrict__ F, const GridDev g,
-                                                       float hc, float c, int chain) {
+__global__ void __launch_bounds__(1024) k_fields_small(float* __restrict__ F, const float* J,
+                                                       const GridDev g, float hc, float c,
+                                                       int chain) {
+  grid_dependency();
+  extern __shared__ float sm[];  // the 9 planes
   const int n0 = g.n[0], n1 = g.n[1];
   const int cells = (int)g.plane;
   for (int t = threadIdx.x; t < cells; t += blockDim.x) {
-    const int i = t % n0, r = t / n0;
-    b_half_point<D>(F, g, i, r % n1, r / n1, hc, 0);
+    float v[9];  // all in flight together
+#pragma unroll
+    for (int q = 0; q < 9; ++q) v[q] = q < 6 ? F[q * cells + t] : J[(q - 6) * cells + t];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) sm[q * cells + t] = v[q];
   }
   __syncthreads();
+  const auto every_point = [&](auto fn) {
+    for (int t = threadIdx.x; t < cells; t += blockDim.x) {
+      const int r = D == 1 ? 0 : t / n0;
+      fn(t - r * n0, D == 3 ? r % n1 : r, D == 3 ? r / n1 : 0);
+    }
+    __syncthreads();
+  };
+  every_point([&](int i, int j, int k) { b_half_point<D>(sm, g, i, j, k, hc, 0); });
+  every_point([&](int i, int j, int k) { e_update_point<D>(sm, sm + 6 * cells, g, i, j, k, c); });
+  if (chain) every_point([&](int i, int j, int k) { b_half_point<D>(sm, g, i, j, k, hc, 1); });
+  const int planes = chain || J != F + JX * g.plane ? 9 : 6;
   for (int t = threadIdx.x; t < cells; t += blockDim.x) {
-    const int i = t % n0, r = t / n0;
-    e_update_point<D>(F, g, i, r % n1, r / n1, c);
-  }
-  if (!chain) return;
-  __syncthreads();
-  for (int t = threadIdx.x; t < cells; t += blockDim.x) {
-    const int i = t % n0, r = t / n0;
-    b_half_point<D>(F, g, i, r % n1, r / n1, hc, 1);
+#pragma unroll
+    for (int q = 0; q < 9; ++q)
+      if (q < planes) F[q * cells + t] = sm[q * cells + t];
   }
 }
 
@@ -137,6 +159,7 @@ __device__ __forceinline__ void arr4(const float4 a, float v[4]) {
 
 template <int D>
 __global__ void k_b_half_x4(float* __restrict__ F, const GridDev g, float hc, int zero_j) {
+  grid_dependency();
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
   const long long P = g.plane;
   const int i = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
@@ -197,7 +220,8 @@ __global__ void k_b_half_x4(float* __restrict__ F, const GridDev g, float hc, in
 }
 
 template <int D>
-__global__ void k_e_update_x4(float* __restrict__ F, const GridDev g, float c) {
+__global__ void k_e_update_x4(float* __restrict__ F, const float* J, const GridDev g, float c) {
+  grid_dependency();
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
   const long long P = g.plane;
   const int i = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
@@ -228,9 +252,9 @@ __global__ void k_e_update_x4(float* __restrict__ F, const GridDev g, float c) {
     arr4(ld4(F + EX * P + idx), ex);
     arr4(ld4(F + EY * P + idx), ey);
     arr4(ld4(F + EZ * P + idx), ez);
-    arr4(ld4(F + JX * P + idx), jx);
-    arr4(ld4(F + JY * P + idx), jy);
-    arr4(ld4(F + JZ * P + idx), jz);
+    arr4(ld4(J + idx), jx);
+    arr4(ld4(J + P + idx), jy);
+    arr4(ld4(J + 2 * P + idx), jz);
 #pragma unroll
     for (int l = 0; l < 4; ++l) {
       float cx = 0.f, cy = 0.f, cz = 0.f;
@@ -251,6 +275,11 @@ __global__ void k_e_update_x4(float* __restrict__ F, const GridDev g, float c) {
     st4(F + EX * P + idx, ex);
     st4(F + EY * P + idx, ey);
     st4(F + EZ * P + idx, ez);
+    if (J != F + JX * P) {
+      st4(F + JX * P + idx, jx);
+      st4(F + JY * P + idx, jy);
+      st4(F + JZ * P + idx, jz);
+    }
   }
 }
 
@@ -301,6 +330,7 @@ __device__ __forceinline__ float d4m(const float* A, long long i, const Nb& b) {
 // FDTD4 versions of the two updates (same structure as above, wider stencil).
 template <int D>
 __global__ void k_b_half4(float* __restrict__ F, const GridDev g, float hc, int zero_j) {
+  grid_dependency();
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
   const long long P = g.plane;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -336,7 +366,8 @@ __global__ void k_b_half4(float* __restrict__ F, const GridDev g, float hc, int 
 }
 
 template <int D>
-__global__ void k_e_update4(float* __restrict__ F, const GridDev g, float c) {
+__global__ void k_e_update4(float* __restrict__ F, const float* J, const GridDev g, float c) {
+  grid_dependency();
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
   const long long P = g.plane;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -360,9 +391,15 @@ __global__ void k_e_update4(float* __restrict__ F, const GridDev g, float c) {
       cx -= d4m(By, idx, nz);
       cy += d4m(Bx, idx, nz);
     }
-    F[EX * P + idx] = fmaf(c, cx, F[EX * P + idx]) - F[JX * P + idx];
-    F[EY * P + idx] = fmaf(c, cy, F[EY * P + idx]) - F[JY * P + idx];
-    F[EZ * P + idx] = fmaf(c, cz, F[EZ * P + idx]) - F[JZ * P + idx];
+    const float jx = J[idx], jy = J[P + idx], jz = J[2 * P + idx];
+    F[EX * P + idx] = fmaf(c, cx, F[EX * P + idx]) - jx;
+    F[EY * P + idx] = fmaf(c, cy, F[EY * P + idx]) - jy;
+    F[EZ * P + idx] = fmaf(c, cz, F[EZ * P + idx]) - jz;
+    if (J != F + JX * P) {
+      F[JX * P + idx] = jx;
+      F[JY * P + idx] = jy;
+      F[JZ * P + idx] = jz;
+    }
   }
 }
 
@@ -381,21 +418,21 @@ cudaError_t launch_b_half(const GridDev& g, float* F, int zero_j, cudaStream_t s
   if (g.order == 2 && x4_ok(g, F)) {
     const RowLaunch L = row_launch_x4(g);
     switch (g.dim) {
-      case 1: k_b_half_x4<1><<<L.grid, L.threads, 0, st>>>(F, g, hc, zero_j); break;
-      case 2: k_b_half_x4<2><<<L.grid, L.threads, 0, st>>>(F, g, hc, zero_j); break;
-      case 3: k_b_half_x4<3><<<L.grid, L.threads, 0, st>>>(F, g, hc, zero_j); break;
+      case 1: launch_kernel(g.pdl, k_b_half_x4<1>, L.grid, L.threads, 0, st, F, g, hc, zero_j); break;
+      case 2: launch_kernel(g.pdl, k_b_half_x4<2>, L.grid, L.threads, 0, st, F, g, hc, zero_j); break;
+      case 3: launch_kernel(g.pdl, k_b_half_x4<3>, L.grid, L.threads, 0, st, F, g, hc, zero_j); break;
       default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
   }
   const RowLaunch L = row_launch(g);
   switch (g.dim * 10 + g.order) {
-    case 12: k_b_half<1><<<L.grid, L.threads, 0, st>>>(F, g, hc, zero_j); break;
-    case 22: k_b_half<2><<<L.grid, L.threads, 0, st>>>(F, g, hc, zero_j); break;
-    case 32: k_b_half<3><<<L.grid, L.threads, 0, st>>>(F, g, hc, zero_j); break;
-    case 14: k_b_half4<1><<<L.grid, L.threads, 0, st>>>(F, g, hc, zero_j); break;
-    case 24: k_b_half4<2><<<L.grid, L.threads, 0, st>>>(F, g, hc, zero_j); break;
-    case 34: k_b_half4<3><<<L.grid, L.threads, 0, st>>>(F, g, hc, zero_j); break;
+    case 12: launch_kernel(g.pdl, k_b_half<1>, L.grid, L.threads, 0, st, F, g, hc, zero_j); break;
+    case 22: launch_kernel(g.pdl, k_b_half<2>, L.grid, L.threads, 0, st, F, g, hc, zero_j); break;
+    case 32: launch_kernel(g.pdl, k_b_half<3>, L.grid, L.threads, 0, st, F, g, hc, zero_j); break;
+    case 14: launch_kernel(g.pdl, k_b_half4<1>, L.grid, L.threads, 0, st, F, g, hc, zero_j); break;
+    case 24: launch_kernel(g.pdl, k_b_half4<2>, L.grid, L.threads, 0, st, F, g, hc, zero_j); break;
+    case 34: launch_kernel(g.pdl, k_b_half4<3>, L.grid, L.threads, 0, st, F, g, hc, zero_j); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -405,36 +442,45 @@ bool fields_small_ok(const GridDev& g) {
   return PIC_SMALL_FIELDS && g.order == 2 && g.plane <= kSmallFieldCells;
 }
 
-cudaError_t launch_fields_small(const GridDev& g, float* F, cudaStream_t st, int chain) {
+cudaError_t launch_fields_small(const GridDev& g, float* F, const float* J, cudaStream_t st,
+                                int chain) {
+  const size_t smem = 9 * sizeof(float) * (size_t)g.plane;
   const int threads = g.plane < 1024 ? (int)((g.plane + 31) / 32 * 32) : 1024;
+  const auto small = [&](auto kernel) {
+    if (smem > 48 * 1024) {
+      const cudaError_t e = cudaFuncSetAttribute(
+          kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 9 * sizeof(float) * kSmallFieldCells);
+      if (e != cudaSuccess) return e;
+    }
+    return launch_kernel(g.pdl, kernel, 1, threads, smem, st, F, J, g, 0.5f * g.c, g.c, chain);
+  };
   switch (g.dim) {
-    case 1: k_fields_small<1><<<1, threads, 0, st>>>(F, g, 0.5f * g.c, g.c, chain); break;
-    case 2: k_fields_small<2><<<1, threads, 0, st>>>(F, g, 0.5f * g.c, g.c, chain); break;
-    case 3: k_fields_small<3><<<1, threads, 0, st>>>(F, g, 0.5f * g.c, g.c, chain); break;
+    case 1: return small(k_fields_small<1>);
+    case 2: return small(k_fields_small<2>);
+    case 3: return small(k_fields_small<3>);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
-cudaError_t launch_e_update(const GridDev& g, float* F, cudaStream_t st) {
-  if (g.order == 2 && x4_ok(g, F)) {
+cudaError_t launch_e_update(const GridDev& g, float* F, const float* J, cudaStream_t st) {
+  if (g.order == 2 && x4_ok(g, F) && (reinterpret_cast<uintptr_t>(J) & 15) == 0) {
     const RowLaunch L = row_launch_x4(g);
     switch (g.dim) {
-      case 1: k_e_update_x4<1><<<L.grid, L.threads, 0, st>>>(F, g, g.c); break;
-      case 2: k_e_update_x4<2><<<L.grid, L.threads, 0, st>>>(F, g, g.c); break;
-      case 3: k_e_update_x4<3><<<L.grid, L.threads, 0, st>>>(F, g, g.c); break;
+      case 1: launch_kernel(g.pdl, k_e_update_x4<1>, L.grid, L.threads, 0, st, F, J, g, g.c); break;
+      case 2: launch_kernel(g.pdl, k_e_update_x4<2>, L.grid, L.threads, 0, st, F, J, g, g.c); break;
+      case 3: launch_kernel(g.pdl, k_e_update_x4<3>, L.grid, L.threads, 0, st, F, J, g, g.c); break;
       default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
   }
   const RowLaunch L = row_launch(g);
   switch (g.dim * 10 + g.order) {
-    case 12: k_e_update<1><<<L.grid, L.threads, 0, st>>>(F, g, g.c); break;
-    case 22: k_e_update<2><<<L.grid, L.threads, 0, st>>>(F, g, g.c); break;
-    case 32: k_e_update<3><<<L.grid, L.threads, 0, st>>>(F, g, g.c); break;
-    case 14: k_e_update4<1><<<L.grid, L.threads, 0, st>>>(F, g, g.c); break;
-    case 24: k_e_update4<2><<<L.grid, L.threads, 0, st>>>(F, g, g.c); break;
-    case 34: k_e_update4<3><<<L.grid, L.threads, 0, st>>>(F, g, g.c); break;
+    case 12: launch_kernel(g.pdl, k_e_update<1>, L.grid, L.threads, 0, st, F, J, g, g.c); break;
+    case 22: launch_kernel(g.pdl, k_e_update<2>, L.grid, L.threads, 0, st, F, J, g, g.c); break;
+    case 32: launch_kernel(g.pdl, k_e_update<3>, L.grid, L.threads, 0, st, F, J, g, g.c); break;
+    case 14: launch_kernel(g.pdl, k_e_update4<1>, L.grid, L.threads, 0, st, F, J, g, g.c); break;
+    case 24: launch_kernel(g.pdl, k_e_update4<2>, L.grid, L.threads, 0, st, F, J, g, g.c); break;
+    case 34: launch_kernel(g.pdl, k_e_update4<3>, L.grid, L.threads, 0, st, F, J, g, g.c); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

@@ -115,6 +115,7 @@ template <int K>
 __global__ void __launch_bounds__(128) k_filter_x1(const float* __restrict__ src,
                                                    float* __restrict__ dst, const GridDev g,
                                                    int vec) {
+  grid_dependency();
   const int lane = threadIdx.x & 31, n0 = g.n[0];
   const long long x0 = ((long long)blockIdx.x * 4 + (threadIdx.x >> 5)) * kOutX;
   if (x0 >= n0) return;
@@ -142,6 +143,7 @@ template <int K>
 __global__ void __launch_bounds__(128) k_filter_y2(const float* __restrict__ src,
                                                    float* __restrict__ dst, const GridDev g,
                                                    int strips, int run, int vec) {
+  grid_dependency();
   __shared__ float4 ring[kRows][128];
   const int lane = threadIdx.x & 31, n0 = g.n[0], n1 = g.n[1];
   const long long w = (long long)blockIdx.x * 4 + (threadIdx.x >> 5);
@@ -243,6 +245,7 @@ __global__ void __launch_bounds__(256, 4) k_filter_z3(const float* __restrict__ 
                                                      float* __restrict__ dst, const GridDev g,
                                                      int ncx, int ncy, int zrun, int vec,
                                                      int* status) {
+  grid_dependency();
   __shared__ __align__(16) float stage[ZS][ZPLANE];
   __shared__ unsigned long long full[ZS];  // BULK: stage's rows have landed
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
@@ -419,6 +422,7 @@ constexpr int YROW = YX + 8;  // stage row: [3] left halo, [4, 4 + YX) interior,
 __global__ void __launch_bounds__(256) k_filter_y2_one(const float* __restrict__ src,
                                                       float* __restrict__ dst, const GridDev g,
                                                       int ncx, int yrun, int* status) {
+  grid_dependency();
   __shared__ __align__(16) float stage[ZS][YROW];
   __shared__ unsigned long long full[ZS];  // the stage's row has landed
   const int n0 = g.n[0], n1 = g.n[1];
@@ -509,6 +513,7 @@ struct Z3Smem {
 __global__ void __launch_bounds__(32 * kWarpsZ, 2)
     k_filter_z3_two(const float* __restrict__ src, float* __restrict__ dst, const GridDev g, int ncx,
                 int ncy, int run, int vec) {
+  grid_dependency();
   extern __shared__ __align__(16) unsigned char smem[];
   Z3Smem& S = *reinterpret_cast<Z3Smem*>(smem);
   constexpr int K = 2, R = kRowsZ, kOutY = kColY - 2 * K;
@@ -630,9 +635,9 @@ static cudaError_t launch_pass_z3(const GridDev& g, const float* src, float* dst
   // bulk row copies where a status word can report a wait that ran out
   const dim3 grid((unsigned)blocks, (unsigned)ncomp);
   if (vec && status)
-    k_filter_z3<true><<<grid, 256, 0, st>>>(src, dst, g, ncx, ncy, zrun, vec, status);
+    launch_kernel(g.pdl, k_filter_z3<true>, grid, 256, 0, st, src, dst, g, ncx, ncy, zrun, vec, status);
   else
-    k_filter_z3<false><<<grid, 256, 0, st>>>(src, dst, g, ncx, ncy, zrun, vec, status);
+    launch_kernel(g.pdl, k_filter_z3<false>, grid, 256, 0, st, src, dst, g, ncx, ncy, zrun, vec, status);
   return cudaGetLastError();
 }
 
@@ -656,8 +661,7 @@ static cudaError_t launch_one_y2(const GridDev& g, const float* src, float* dst,
   const int yrun = (int)((g.n[1] + runs - 1) / runs);
   const long long blocks = (long long)ncx * ((g.n[1] + yrun - 1) / yrun);
   if (blocks > 0x7fffffffLL || ncomp > 65535) return cudaErrorInvalidValue;
-  k_filter_y2_one<<<dim3((unsigned)blocks, (unsigned)ncomp), 256, 0, st>>>(src, dst, g, ncx, yrun,
-                                                                            status);
+  launch_kernel(g.pdl, k_filter_y2_one, dim3((unsigned)blocks, (unsigned)ncomp), 256, 0, st, src, dst, g, ncx, yrun, status);
   return cudaGetLastError();
 }
 
@@ -676,8 +680,7 @@ static cudaError_t launch_two_z3(const GridDev& g, const float* src, float* dst,
   const cudaError_t e = cudaFuncSetAttribute(
       k_filter_z3_two, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Z3Smem));
   if (e != cudaSuccess) return e;
-  k_filter_z3_two<<<dim3((unsigned)blocks, ncomp), 32 * kWarpsZ, sizeof(Z3Smem), st>>>(
-      src, dst, g, ncx, ncy, run, vec);
+  launch_kernel(g.pdl, k_filter_z3_two, dim3((unsigned)blocks, ncomp), 32 * kWarpsZ, sizeof(Z3Smem), st, src, dst, g, ncx, ncy, run, vec);
   return cudaGetLastError();
 }
 
@@ -688,7 +691,7 @@ static cudaError_t launch_k(const GridDev& g, const float* src, float* dst, int 
   const int sms = device_sms();
   const long long strips = ((long long)g.n[0] + kOutX - 1) / kOutX;
   if (g.dim == 1) {
-    k_filter_x1<K><<<dim3((unsigned)((strips + 3) / 4), ncomp), 128, 0, st>>>(src, dst, g, vec);
+    launch_kernel(g.pdl, k_filter_x1<K>, dim3((unsigned)((strips + 3) / 4), ncomp), 128, 0, st, src, dst, g, vec);
   } else if (g.dim == 2) {
     // runs short enough for 16 warps per SM, but no shorter than the K rows
     // of halo on either side
@@ -696,8 +699,7 @@ static cudaError_t launch_k(const GridDev& g, const float* src, float* dst, int 
     long long run = (g.n[1] * strips * ncomp + warps - 1) / warps;
     run = run < 2 * K ? 2 * K : run;
     const long long runs = (g.n[1] + run - 1) / run;
-    k_filter_y2<K><<<dim3((unsigned)((strips * runs + 3) / 4), ncomp), 128, 0, st>>>(
-        src, dst, g, (int)strips, (int)run, vec);
+    launch_kernel(g.pdl, k_filter_y2<K>, dim3((unsigned)((strips * runs + 3) / 4), ncomp), 128, 0, st, src, dst, g, (int)strips, (int)run, vec);
   }
   return cudaGetLastError();
 }

@@ -151,6 +151,26 @@ inline RowLaunch row_launch(const GridDev& g) {
   return {dim3((unsigned)((n0 + t - 1) / t), gy, gz), t};
 }
 
+// Kernel launch; with pdl (programmatic dependent launch) the kernel may be set
+// up on the SMs while the one before it on the stream still runs, and its
+// grid_dependency() holds it until that one is complete.  Only for kernels
+// that call grid_dependency() before anything else.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_kernel(int pdl, void (*kernel)(KArgs...), dim3 grid, dim3 block,
+                                 size_t smem, cudaStream_t st, const Args&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 struct PushParams {
   GridDev g;
   TileDev t;
@@ -205,13 +225,16 @@ size_t particle_smem_bytes(int dim, const TileDev& t);
 long long window_landing_floats(int dim, const TileDev& t);
 
 cudaError_t launch_b_half(const GridDev& g, float* F, int zero_j, cudaStream_t st);
-cudaError_t launch_e_update(const GridDev& g, float* F, cudaStream_t st);
+// J: the three current planes, F's own or the filter's buffer (then also
+// copied to F's)
+cudaError_t launch_e_update(const GridDev& g, float* F, const float* J, cudaStream_t st);
 // FDTD2 lattices of at most kSmallFieldCells points: the second B half step
 // and the E update in one single-block launch (the same bits as the two);
 // with chain != 0 also the next step's first B half step (clearing J)
 constexpr long long kSmallFieldCells = 4096;
 bool fields_small_ok(const GridDev& g);
-cudaError_t launch_fields_small(const GridDev& g, float* F, cudaStream_t st, int chain = 0);
+cudaError_t launch_fields_small(const GridDev& g, float* F, const float* J, cudaStream_t st,
+                                int chain = 0);
 // `passes` Binomial2 passes (up to 4, in 3D up to 2) over ncomp consecutive
 // planes, src -> dst (src != dst), in one launch, and how many such launches
 // p passes take.  With a status word, 3D rows are staged by bulk copies whose
@@ -237,7 +260,7 @@ cudaError_t launch_tile_count(const SortParams& P, const int* cell, long long n,
 // exclusive scan of count[0..n) into start[0..n] and cursor; n above 4096 uses
 // scratch (scan_scratch(n) ints)
 cudaError_t launch_tile_scan(const int* count, int ntiles, int* start, int* cursor, int* scratch,
-                             cudaStream_t st);
+                             cudaStream_t st, int pdl);
 inline long long scan_scratch(long long n) { return 3 * ((n + 4095) / 4096 + 1); }
 // arrays with rows of ld elements, the first n of which are particles
 // perm (or null): perm[new slot] = old slot
@@ -251,7 +274,7 @@ cudaError_t launch_tile_scatter(const SortParams& P, const int* cell, const floa
 cudaError_t launch_clip_starts(const int* tstart, long long nb1, int lo, int hi, int* out,
                                cudaStream_t st);
 cudaError_t launch_check_buckets(int* tstart, long long nb, long long n, int* status,
-                                 cudaStream_t st);
+                                 cudaStream_t st, int pdl);
 // out[r * ld + perm[i]] = in[r * ld + i] for i < n, r < rows (entries of perm
 // outside [0, n) skipped, ST_BAD_BUCKETS set)
 cudaError_t launch_unpermute(const int* perm, const float* in, float* out, long long n,

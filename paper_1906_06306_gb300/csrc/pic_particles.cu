@@ -424,6 +424,7 @@ __global__ void __launch_bounds__(kPushThreads, D == 3 ? PIC_PUSH_MIN_BLOCKS_3D
                                                 : TMA  ? PIC_PUSH_MIN_BLOCKS_TMA
                                                        : PIC_PUSH_MIN_BLOCKS)
     k_particles(const __grid_constant__ PushParams P) {
+  grid_dependency();
   extern __shared__ __align__(128) float sm[];
   static_assert(!TMA || D < 3, "the record stream is for the 1D/2D kernels");
   constexpr int NR = 1 + D + 3;  // record rows: cell, D offsets, 3 four-velocity components
@@ -835,6 +836,7 @@ __global__ void __launch_bounds__(kPushThreads, D == 3 ? PIC_PUSH_MIN_BLOCKS_3D
 // yet: they take the global-memory path, grid-strided over [tail, n).
 template <int D>
 __global__ void __launch_bounds__(kPushThreads) k_particles_tail(const PushParams P) {
+  grid_dependency();
   const GlobAcc GA{P.F, P.g.plane, P.g.n[0], P.g.n[1], P.g.n[2]};
   for (int s = 0; s < P.nspecies; ++s) {
     const SpeciesDev& S = P.sp[s];
@@ -853,6 +855,7 @@ __global__ void __launch_bounds__(kPushThreads) k_particles_tail(const PushParam
 // where k_particles read them; each slot is listed at most once per launch.
 template <int D, int MODE>
 __global__ void __launch_bounds__(kPushThreads) k_particles_deferred(const PushParams P) {
+  grid_dependency();
   const GlobAcc GA{P.F, P.g.plane, P.g.n[0], P.g.n[1], P.g.n[2]};
   for (int s = 0; s < P.nspecies; ++s) {
     const SpeciesDev& S = P.sp[s];
@@ -946,6 +949,16 @@ cudaError_t set_particle_smem_limit(int bytes) {
 template <int D, int MODE>
 static cudaError_t launch(const PushParams& P, cudaStream_t st) {
   const unsigned nblocks = (unsigned)P.t.ntiles * (unsigned)P.splits;
+  // Blocks placed while the last kernel's are still on the SMs are spread less
+  // evenly.  Where all blocks run in one wave and are long (from 2048 particles
+  // on) the fullest SM decides, and that costs more than the early set-up
+  // gains: 133^2 box, 648 blocks of 2184 particles, 20 steps 1055 us with,
+  // 1008 without; 130 x 94 box, 648 blocks of 300, a step 29.0 with, 31.3
+  // without; 128^2 box, 640 blocks of 1640, gradient 5.45 ms with, 5.55 without.
+  long long ntot = 0;
+  for (int s = 0; s < P.nspecies; ++s) ntot += P.sp[s].n;
+  const unsigned wave = 152u * (D == 3 ? PIC_PUSH_MIN_BLOCKS_3D : PIC_PUSH_MIN_BLOCKS);
+  const int pdl = P.g.pdl && !(nblocks <= wave && ntot >= 2048LL * nblocks);
   // the deferred lists can have entries in 3D (strays) and with the wall
   constexpr bool deferred = D == 3 || MODE == 3;
   if (deferred) {
@@ -963,30 +976,30 @@ static cudaError_t launch(const PushParams& P, cudaStream_t st) {
   constexpr bool kStreamable = PIC_TMA_RECORDS && D < 3 && (MODE == 0 || MODE == 3);
   const bool tma = kStreamable && P.rec_aligned;
   if (D == 2 && MODE == 0 && P.t.W[0] == 23 && P.t.W[1] == 15 && tma)
-    k_particles<2, 0, 23, 15, 1, kStreamable><<<nblocks, kPushThreads, smem, st>>>(P);
+    launch_kernel(pdl, k_particles<2, 0, 23, 15, 1, kStreamable>, nblocks, kPushThreads, smem, st, P);
   else if (D == 2 && MODE == 0 && P.t.W[0] == 23 && P.t.W[1] == 23 && tma)
-    k_particles<2, 0, 23, 23, 1, kStreamable><<<nblocks, kPushThreads, smem, st>>>(P);
+    launch_kernel(pdl, k_particles<2, 0, 23, 23, 1, kStreamable>, nblocks, kPushThreads, smem, st, P);
   else if (D == 2 && MODE == 0 && P.t.W[0] == 23 && P.t.W[1] == 15)
-    k_particles<2, 0, 23, 15><<<nblocks, kPushThreads, smem, st>>>(P);
+    launch_kernel(pdl, k_particles<2, 0, 23, 15>, nblocks, kPushThreads, smem, st, P);
   else if (D == 2 && MODE == 0 && P.t.W[0] == 23 && P.t.W[1] == 23)
-    k_particles<2, 0, 23, 23><<<nblocks, kPushThreads, smem, st>>>(P);
+    launch_kernel(pdl, k_particles<2, 0, 23, 23>, nblocks, kPushThreads, smem, st, P);
   else if (D == 2 && MODE == 0 && P.t.W[0] == 25 && P.t.W[1] == 17)
-    k_particles<2, 0, 25, 17><<<nblocks, kPushThreads, smem, st>>>(P);
+    launch_kernel(pdl, k_particles<2, 0, 25, 17>, nblocks, kPushThreads, smem, st, P);
   else if (tma)
-    k_particles<D, MODE, 0, 0, 1, kStreamable><<<nblocks, kPushThreads, smem, st>>>(P);
+    launch_kernel(pdl, k_particles<D, MODE, 0, 0, 1, kStreamable>, nblocks, kPushThreads, smem, st, P);
   else if (D == 3 && MODE == 0 && w3)
-    k_particles<3, 0, 13, 13, 9><<<nblocks, kPushThreads, smem, st>>>(P);
+    launch_kernel(pdl, k_particles<3, 0, 13, 13, 9>, nblocks, kPushThreads, smem, st, P);
   else if (D == 3 && MODE == 3 && w3)
-    k_particles<3, 3, 13, 13, 9><<<nblocks, kPushThreads, smem, st>>>(P);
+    launch_kernel(pdl, k_particles<3, 3, 13, 13, 9>, nblocks, kPushThreads, smem, st, P);
   else if (D == 3 && MODE == 0 && w37)
-    k_particles<3, 0, 13, 13, 7><<<nblocks, kPushThreads, smem, st>>>(P);
+    launch_kernel(pdl, k_particles<3, 0, 13, 13, 7>, nblocks, kPushThreads, smem, st, P);
   else if (D == 3 && MODE == 3 && w37)
-    k_particles<3, 3, 13, 13, 7><<<nblocks, kPushThreads, smem, st>>>(P);
+    launch_kernel(pdl, k_particles<3, 3, 13, 13, 7>, nblocks, kPushThreads, smem, st, P);
   else
-    k_particles<D, MODE><<<nblocks, kPushThreads, smem, st>>>(P);
+    launch_kernel(pdl, k_particles<D, MODE>, nblocks, kPushThreads, smem, st, P);
   if ((MODE == 0 || MODE == 3) && P.tail_blocks > 0)
-    k_particles_tail<D><<<(unsigned)P.tail_blocks, kPushThreads, 0, st>>>(P);
-  if (deferred) k_particles_deferred<D, MODE><<<4 * 152, kPushThreads, 0, st>>>(P);
+    launch_kernel(P.g.pdl, k_particles_tail<D>, (unsigned)P.tail_blocks, kPushThreads, 0, st, P);
+  if (deferred) launch_kernel(P.g.pdl, k_particles_deferred<D, MODE>, 4 * 152, kPushThreads, 0, st, P);
   return cudaSuccess;
 }
 

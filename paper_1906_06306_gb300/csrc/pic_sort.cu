@@ -34,9 +34,10 @@ __device__ __forceinline__ int tile_key(const SortParams& P, int cell) {
     tile = tile * P.t.nt[d] + t;
     x[d] -= t * P.t.T[d];
   }
-  if (D == 1) return tile;  // 1D tiles are not subdivided
+  if constexpr (D > 1) {  // 1D tiles are not subdivided
 #pragma unroll
-  for (int d = D - 1; d >= 0; --d) sub = sub * P.t.ns[d] + fdiv(x[d], *ds[d]);
+    for (int d = D - 1; d >= 0; --d) sub = sub * P.t.ns[d] + fdiv(x[d], *ds[d]);
+  }
   return tile * P.t.nsub + sub;
 }
 
@@ -65,6 +66,7 @@ constexpr int kCountSlots = 1024;
 template <int D>
 __global__ void __launch_bounds__(256) k_tile_count(const SortParams P, const int* __restrict__ cell,
                                                     long long n, long long chunk, int* count) {
+  grid_dependency();
   __shared__ int skey[kCountSlots];
   __shared__ int scnt[kCountSlots];
   for (int s = threadIdx.x; s < kCountSlots; s += blockDim.x) {
@@ -105,6 +107,7 @@ __global__ void __launch_bounds__(256) k_tile_count(const SortParams P, const in
 // total) and cursor = start, in one block of 1024 threads.
 __global__ void __launch_bounds__(1024) k_tile_scan(const int* __restrict__ count, int ntiles,
                                                     int* start, int* cursor) {
+  grid_dependency();
   __shared__ int warp_sums[32];
   __shared__ int carry;
   if (threadIdx.x == 0) carry = 0;
@@ -150,6 +153,7 @@ __global__ void __launch_bounds__(1024) k_tile_scan(const int* __restrict__ coun
 constexpr int kScanChunk = 4096;  // counts per block: 4 per thread of 1024
 __global__ void __launch_bounds__(1024) k_scan_chunks(const int* __restrict__ count, int n,
                                                       int* start, int* part) {
+  grid_dependency();
   __shared__ int warp_sums[32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int base = blockIdx.x * kScanChunk + 4 * threadIdx.x;
@@ -188,6 +192,7 @@ __global__ void __launch_bounds__(1024) k_scan_chunks(const int* __restrict__ co
 
 __global__ void __launch_bounds__(1024) k_scan_add(int* start, int* cursor, int n,
                                                    const int* part_scan) {
+  grid_dependency();
   const int off = part_scan[blockIdx.x];
   const int base = blockIdx.x * kScanChunk + 4 * threadIdx.x;
 #pragma unroll
@@ -207,6 +212,7 @@ __global__ void k_tile_scatter_lanes(const SortParams P, const int* __restrict__
                                long long n, long long ld, int* cursor, int* __restrict__ cell_out,
                                float* __restrict__ off_out, float* __restrict__ u_out,
                                int* __restrict__ perm) {
+  grid_dependency();
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long base = (long long)blockIdx.x * blockDim.x; base < n; base += stride) {
     const long long p = base + threadIdx.x;
@@ -241,6 +247,7 @@ __global__ void __launch_bounds__(256) k_tile_scatter(
     const SortParams P, const int* __restrict__ cell, const float* __restrict__ off,
     const float* __restrict__ u, long long n, long long ld, int* cursor, int* __restrict__ cell_out,
     float* __restrict__ off_out, float* __restrict__ u_out, int* __restrict__ perm) {
+  grid_dependency();
   constexpr int kChunk = 256 * U;
   __shared__ int skey[kCountSlots];  // bin of a table slot, then the bin's reserved global slot
   __shared__ int scnt[kCountSlots];  // its particles here, then their first place in bin order
@@ -376,6 +383,7 @@ static unsigned blocks_for(long long n) {
 cudaError_t launch_tile_count(const SortParams& P, const int* cell, long long n, int* count,
                               cudaStream_t st) {
   if (n == 0) return cudaSuccess;
+  const int pdl = P.g.pdl;
   // contiguous chunks of at least 4096 particles (a multiple of 256), at most
   // 16 blocks per SM
   long long nb = (n + 4095) / 4096;
@@ -383,18 +391,18 @@ cudaError_t launch_tile_count(const SortParams& P, const int* cell, long long n,
   const long long chunk = ((n + nb - 1) / nb + 255) / 256 * 256;
   nb = (n + chunk - 1) / chunk;
   switch (P.g.dim) {
-    case 1: k_tile_count<1><<<(unsigned)nb, 256, 0, st>>>(P, cell, n, chunk, count); break;
-    case 2: k_tile_count<2><<<(unsigned)nb, 256, 0, st>>>(P, cell, n, chunk, count); break;
-    case 3: k_tile_count<3><<<(unsigned)nb, 256, 0, st>>>(P, cell, n, chunk, count); break;
+    case 1: launch_kernel(pdl, k_tile_count<1>, (unsigned)nb, 256, 0, st, P, cell, n, chunk, count); break;
+    case 2: launch_kernel(pdl, k_tile_count<2>, (unsigned)nb, 256, 0, st, P, cell, n, chunk, count); break;
+    case 3: launch_kernel(pdl, k_tile_count<3>, (unsigned)nb, 256, 0, st, P, cell, n, chunk, count); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
 }
 
 cudaError_t launch_tile_scan(const int* count, int ntiles, int* start, int* cursor, int* scratch,
-                             cudaStream_t st) {
+                             cudaStream_t st, int pdl) {
   if (ntiles <= kScanChunk) {
-    k_tile_scan<<<1, 1024, 0, st>>>(count, ntiles, start, cursor);
+    launch_kernel(pdl, k_tile_scan, 1, 1024, 0, st, count, ntiles, start, cursor);
     return cudaGetLastError();
   }
   // scratch: block totals [nb], their scan [nb + 1], the scan's cursor [nb]
@@ -402,9 +410,9 @@ cudaError_t launch_tile_scan(const int* count, int ntiles, int* start, int* curs
   int* part = scratch;
   int* part_scan = scratch + nb;
   int* part_cursor = scratch + 2 * nb + 1;
-  k_scan_chunks<<<nb, 1024, 0, st>>>(count, ntiles, start, part);
-  k_tile_scan<<<1, 1024, 0, st>>>(part, nb, part_scan, part_cursor);
-  k_scan_add<<<nb, 1024, 0, st>>>(start, cursor, ntiles, part_scan);
+  launch_kernel(pdl, k_scan_chunks, nb, 1024, 0, st, count, ntiles, start, part);
+  launch_kernel(pdl, k_tile_scan, 1, 1024, 0, st, part, nb, part_scan, part_cursor);
+  launch_kernel(pdl, k_scan_add, nb, 1024, 0, st, start, cursor, ntiles, part_scan);
   return cudaGetLastError();
 }
 
@@ -413,10 +421,10 @@ cudaError_t launch_tile_scatter(const SortParams& P, const int* cell, const floa
                                 int* cell_out, float* off_out, float* u_out, cudaStream_t st,
                                 int* perm) {
   if (n == 0) return cudaSuccess;
+  const int pdl = P.g.pdl;
   const auto launch = [&](auto kernel, int chunk) {
-    kernel<<<(unsigned)((n + chunk - 1) / chunk), 256, 0, st>>>(P, cell, off, u, n, ld, cursor, cell_out,
-                                                                off_out, u_out, perm);
-    return cudaGetLastError();
+    return launch_kernel(pdl, kernel, (unsigned)((n + chunk - 1) / chunk), 256, 0, st, P, cell, off, u,
+                         n, ld, cursor, cell_out, off_out, u_out, perm);
   };
   // few particles: the lanes kernel, whose blocks of 256 spread them over more
   // of the chip (65,536 2D particles, whole sort: 70 us against 78 with 1024 to
@@ -424,11 +432,9 @@ cudaError_t launch_tile_scatter(const SortParams& P, const int* cell, const floa
   const bool few = n < 1 << 17, some = n < 1 << 19;
   const unsigned nb = blocks_for(n);
 #define PIC_SCATTER(D)                                                                        \
-  if (few) {                                                                                  \
-    k_tile_scatter_lanes<D><<<nb, 256, 0, st>>>(P, cell, off, u, n, ld, cursor, cell_out,     \
-                                                off_out, u_out, perm);                        \
-    return cudaGetLastError();                                                                \
-  }                                                                                           \
+  if (few)                                                                                    \
+    return launch_kernel(pdl, k_tile_scatter_lanes<D>, nb, 256, 0, st, P, cell, off, u, n, ld, \
+                         cursor, cell_out, off_out, u_out, perm);                             \
   return some ? launch(k_tile_scatter<D, 4>, 1024) : launch(k_tile_scatter<D, 8>, 2048);
   switch (P.g.dim) {
     case 1: PIC_SCATTER(1)
@@ -444,6 +450,7 @@ cudaError_t launch_tile_scatter(const SortParams& P, const int* cell, const floa
 // bucket: the last tile's blocks take every particle, all through the stray
 // path) and the status word says so.
 __global__ void k_check_buckets(int* __restrict__ t, long long nb, long long n, int* status) {
+  grid_dependency();
   bool bad = threadIdx.x == 0 && (t[0] != 0 || t[nb] != n);
   for (long long i = threadIdx.x; i < nb; i += blockDim.x) bad |= t[i] > t[i + 1];
   if (!__syncthreads_or(bad)) return;
@@ -455,8 +462,8 @@ __global__ void k_check_buckets(int* __restrict__ t, long long nb, long long n, 
 }
 
 cudaError_t launch_check_buckets(int* tstart, long long nb, long long n, int* status,
-                                 cudaStream_t st) {
-  k_check_buckets<<<1, 1024, 0, st>>>(tstart, nb, n, status);
+                                 cudaStream_t st, int pdl) {
+  launch_kernel(pdl, k_check_buckets, 1, 1024, 0, st, tstart, nb, n, status);
   return cudaGetLastError();
 }
 
