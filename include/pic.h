@@ -101,7 +101,7 @@ typedef struct {
  * Binomial2 passes applied to J inside pic_step (Sect. 4.2 uses 8, the
  * 3D shock-shaped workload 4); chunk: target particles per thread block (a box
  * with fewer tiles than 4 per SM splits them further, down to 256 particles
- * per block, until the particle launch has 4 blocks per SM). */
+ * per block, until the blocks of the particle launch fill the GPU). */
 typedef struct {
   int tile[3];
   int halo;
