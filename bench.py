@@ -1133,12 +1133,12 @@ def run_adjoint(args):
     adj_ms, adj_n = kt["adjoint"]
     avg_adj = adj_ms * 1e-3 / max(adj_n, 1)
     # kernels behind the library's timed calls: a push is the tile kernel (2D,
-    # periodic: no deferred-particle kernel), an adjoint step (tile pass) the B
-    # rebuild, 2 adjoint B half steps, the adjoint E update, the filter's
-    # launches, a bucket check per species, the tile pass and the deferred pass
+    # periodic: no deferred-particle kernel), an adjoint step (tile pass) the
+    # bucket starts, the fields it begins with, 2 adjoint B half steps, the
+    # filter's launches, the tile pass and the deferred pass
     passes = sim.tuning()["filter_passes"] - fused_away(sim)
     launches = (kt["push"][1] + kt["b_half"][1] + kt["e_update"][1] + kt["filter"][1] +
-                kt["sort"][1] + (6 + passes + sim.nspecies) * kt["adjoint"][1])
+                kt["sort"][1] + (6 + passes) * kt["adjoint"][1])
     # per adjoint step: particle state read (4 + 8 + 12 B) and gradients read and
     # written (2 x (8 + 12) B); E, B read and their gradients added once per cell
     alg = npart * (24 + 40) + pl.ncells * 4 * (6 + 9 + 12)

@@ -22,9 +22,36 @@
 
 namespace pic {
 
-// Adjoint of E' = E + c curl- B2 - Jf:  Bbar += c curl+ Ebar,  Jbar = -Ebar.
+// curl+ (forward differences) of the planes at X, Y, Z = E, E + P, E + 2 P at
+// point idx, whose upper neighbours are sx, sy, sz away.
 template <int D>
-__global__ void k_adj_e(float* __restrict__ A, const GridDev g, float c) {
+__device__ __forceinline__ void curl_up(const float* E, long long P, long long idx, long long sx,
+                                        long long sy, long long sz, float* e, float* c) {
+  const float *Ex = E, *Ey = E + P, *Ez = E + 2 * P;
+  const float ex = Ex[idx], ey = Ey[idx], ez = Ez[idx];
+  float cx = 0.f, cy = 0.f, cz = 0.f;
+  cy -= Ez[idx + sx] - ez;
+  cz += Ey[idx + sx] - ey;
+  if (D >= 2) {
+    cx += Ez[idx + sy] - ez;
+    cz -= Ex[idx + sy] - ex;
+  }
+  if (D >= 3) {
+    cx -= Ey[idx + sz] - ey;
+    cy += Ex[idx + sz] - ex;
+  }
+  e[0] = ex, e[1] = ey, e[2] = ez;
+  c[0] = cx, c[1] = cy, c[2] = cz;
+}
+
+// What a reverse step begins with, point by point in one launch (a copy and
+// two kernels before: at 128^2 each took longer to launch than to run): the
+// fields that the forward step's particles saw, E and B - (c/2) curl+ E (the
+// operations of the forward half step), from F into F1; and the adjoint of
+// E' = E + c curl- B2 - Jf:  Bbar += c curl+ Ebar,  Jbar = -Ebar.
+template <int D>
+__global__ void k_adj_begin(const float* __restrict__ F, float* __restrict__ F1,
+                            float* __restrict__ A, const GridDev g, float c) {
   grid_dependency();
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
   const long long P = g.plane;
@@ -35,34 +62,27 @@ __global__ void k_adj_e(float* __restrict__ A, const GridDev g, float c) {
     const long long sx = (i + 1 < n0) ? 1 : 1 - n0;
     const long long sy = (D >= 2) ? ((j + 1 < n1) ? n0 : (long long)n0 * (1 - n1)) : 0;
     const long long sz = (D >= 3) ? ((k + 1 < n2) ? (long long)n0 * n1 : (long long)n0 * n1 * (1 - n2)) : 0;
-    const float* Ex = A + EX * P;
-    const float* Ey = A + EY * P;
-    const float* Ez = A + EZ * P;
-    const float ex = Ex[idx], ey = Ey[idx], ez = Ez[idx];
-    float cx = 0.f, cy = 0.f, cz = 0.f;
-    cy -= Ez[idx + sx] - ez;
-    cz += Ey[idx + sx] - ey;
-    if (D >= 2) {
-      cx += Ez[idx + sy] - ez;
-      cz -= Ex[idx + sy] - ex;
+    float e[3], r[3];
+    curl_up<D>(F + EX * P, P, idx, sx, sy, sz, e, r);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      F1[(EX + a) * P + idx] = e[a];
+      F1[(BX + a) * P + idx] = fmaf(-0.5f * c, r[a], F[(BX + a) * P + idx]);
     }
-    if (D >= 3) {
-      cx -= Ey[idx + sz] - ey;
-      cy += Ex[idx + sz] - ex;
+    curl_up<D>(A + EX * P, P, idx, sx, sy, sz, e, r);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      A[(BX + a) * P + idx] += c * r[a];
+      A[(JX + a) * P + idx] = -e[a];
     }
-    A[BX * P + idx] += c * cx;
-    A[BY * P + idx] += c * cy;
-    A[BZ * P + idx] += c * cz;
-    A[JX * P + idx] = -ex;
-    A[JY * P + idx] = -ey;
-    A[JZ * P + idx] = -ez;
   }
 }
 
 // Adjoint of B <- B - h curl+ E (a half step, h = c/2):  Ebar -= h curl- Bbar.
-// Reads only B planes and writes only E planes, so the points are independent.
+// Reads only B planes and writes only E planes (and, asked to, clears J), so the
+// points are independent.
 template <int D>
-__global__ void k_adj_b(float* __restrict__ A, const GridDev g, float h) {
+__global__ void k_adj_b(float* __restrict__ A, const GridDev g, float h, int zero_j) {
   grid_dependency();
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
   const long long P = g.plane;
@@ -91,6 +111,11 @@ __global__ void k_adj_b(float* __restrict__ A, const GridDev g, float h) {
     A[EX * P + idx] -= h * cx;
     A[EY * P + idx] -= h * cy;
     A[EZ * P + idx] -= h * cz;
+    if (zero_j) {
+      A[JX * P + idx] = 0.f;
+      A[JY * P + idx] = 0.f;
+      A[JZ * P + idx] = 0.f;
+    }
   }
 }
 
@@ -581,11 +606,18 @@ __global__ void __launch_bounds__(256, D == 3 ? 2 : PIC_ADJ_MIN_BLOCKS)
       }
       __syncthreads();
       if (mb != 0u) {
-        for (int w = threadIdx.x; w < 6 * ws; w += blockDim.x) {
-          const int v = wi[w];
-          if (v != 0) {
-            wf[w] += (float)v * q;
-            wi[w] = 0;
+        int4* i4 = reinterpret_cast<int4*>(wi);
+        float4* f4 = reinterpret_cast<float4*>(wf);
+        for (int w = threadIdx.x; w < 6 * ws / 4; w += blockDim.x) {
+          const int4 v = i4[w];
+          if ((v.x | v.y | v.z | v.w) != 0) {
+            float4 f = f4[w];
+            f.x += (float)v.x * q;
+            f.y += (float)v.y * q;
+            f.z += (float)v.z * q;
+            f.w += (float)v.w * q;
+            f4[w] = f;
+            i4[w] = make_int4(0, 0, 0, 0);
           }
         }
       }
@@ -603,27 +635,26 @@ __global__ void __launch_bounds__(256, D == 3 ? 2 : PIC_ADJ_MIN_BLOCKS)
   }
 }
 
-cudaError_t launch_adj_e(const GridDev& g, float* A, cudaStream_t st) {
+cudaError_t launch_adj_begin(const GridDev& g, const float* F, float* F1, float* A,
+                             cudaStream_t st) {
   const RowLaunch L = row_launch(g);
   switch (g.dim) {
-    case 1: launch_kernel(g.pdl, k_adj_e<1>, L.grid, L.threads, 0, st, A, g, g.c); break;
-    case 2: launch_kernel(g.pdl, k_adj_e<2>, L.grid, L.threads, 0, st, A, g, g.c); break;
-    case 3: launch_kernel(g.pdl, k_adj_e<3>, L.grid, L.threads, 0, st, A, g, g.c); break;
+    case 1: return launch_kernel(g.pdl, k_adj_begin<1>, L.grid, L.threads, 0, st, F, F1, A, g, g.c);
+    case 2: return launch_kernel(g.pdl, k_adj_begin<2>, L.grid, L.threads, 0, st, F, F1, A, g, g.c);
+    case 3: return launch_kernel(g.pdl, k_adj_begin<3>, L.grid, L.threads, 0, st, F, F1, A, g, g.c);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
-cudaError_t launch_adj_b_half(const GridDev& g, float* A, cudaStream_t st) {
+cudaError_t launch_adj_b_half(const GridDev& g, float* A, int zero_j, cudaStream_t st) {
   const RowLaunch L = row_launch(g);
   const float h = 0.5f * g.c;
   switch (g.dim) {
-    case 1: launch_kernel(g.pdl, k_adj_b<1>, L.grid, L.threads, 0, st, A, g, h); break;
-    case 2: launch_kernel(g.pdl, k_adj_b<2>, L.grid, L.threads, 0, st, A, g, h); break;
-    case 3: launch_kernel(g.pdl, k_adj_b<3>, L.grid, L.threads, 0, st, A, g, h); break;
+    case 1: return launch_kernel(g.pdl, k_adj_b<1>, L.grid, L.threads, 0, st, A, g, h, zero_j);
+    case 2: return launch_kernel(g.pdl, k_adj_b<2>, L.grid, L.threads, 0, st, A, g, h, zero_j);
+    case 3: return launch_kernel(g.pdl, k_adj_b<3>, L.grid, L.threads, 0, st, A, g, h, zero_j);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 // shared memory of the tile pass: 9 float planes (E, B1, current adjoint),
@@ -642,8 +673,7 @@ cudaError_t launch_adj_particles(const AdjParams& P, cudaStream_t st) {
   if (tiled) {
     static bool attr[4] = {false, false, false, false};
     const size_t smem = adj_tile_smem_bytes(P.t);
-    cudaError_t e = cudaMemsetAsync(P.dcount, 0, sizeof(int) * P.nspecies, st);
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
     if (!attr[D]) {
       const void* k1 = D == 1 ? (const void*)k_adj_tiles<1> : D == 2 ? (const void*)k_adj_tiles<2>
                                                                       : (const void*)k_adj_tiles<3>;

@@ -517,6 +517,26 @@ cudaError_t sort_species(pic_ctx* ctx, int s, bool copy_back, int32_t* perm) {
   return copy_rows(ctx->sp[s].u, u_out, sizeof(float), n, ld, 3, k, ctx->st);
 }
 
+// Bucket starts handed in from outside, copied and checked (every species with
+// BC.src); clears the deferred lists' counts.  One launch for up to 2^15 bins;
+// one block per species would be long at more (a checkpoint's step of a 256^2
+// box 84 -> 80 us, the launches of a copy and a check per species before).
+cudaError_t adopt_buckets(pic_ctx* ctx, const BucketCopies& BC) {
+  const long long nb = sort_bins(ctx->tile);
+  if (nb <= 1 << 15)
+    return launch_adopt_buckets(BC, ctx->ns, nb, ctx->d_dcount, ctx->d_status, ctx->st, ctx->g.pdl);
+  cudaError_t r = cudaMemsetAsync(ctx->d_dcount, 0, sizeof(int) * ctx->ns, ctx->st);
+  for (int s = 0; s < ctx->ns; ++s) {
+    if (!BC.src[s]) continue;
+    if (r == cudaSuccess)
+      r = cudaMemcpyAsync(BC.dst[s], BC.src[s], sizeof(int) * (nb + 1), cudaMemcpyDeviceToDevice,
+                          ctx->st);
+    if (r == cudaSuccess)
+      r = launch_check_buckets(BC.dst[s], nb, BC.n[s], ctx->d_status, ctx->st, ctx->g.pdl);
+  }
+  return r;
+}
+
 // The context's bookkeeping of a tile sort of every species (at the current
 // step, with or without copy back); launches nothing.
 void sort_done(pic_ctx* ctx, bool copy_back) {
@@ -938,7 +958,6 @@ pic_status pic_adjoint_step(pic_ctx* ctx, const float* fwd_fields, const pic_adj
   if (!fwd_fields || !sp || !adj_fields) return set_err(ctx, PIC_ERR_ARG, "NULL argument");
   if (ctx->g.order != 2 || ctx->pusher != PIC_PUSHER_BORIS || ctx->shock)
     return set_err(ctx, PIC_ERR_STATE, "the adjoint covers FDTD2, Boris and periodic boxes");
-  const int D = ctx->grid.dim;
   for (int s = 0; s < ctx->ns; ++s)
     if (ctx->sp[s].n > 0 && (!sp[s].cell || !sp[s].off || !sp[s].u || !sp[s].xbar || !sp[s].ubar))
       return set_err(ctx, PIC_ERR_ARG, "adjoint species buffers are NULL");
@@ -969,15 +988,16 @@ pic_status pic_adjoint_step(pic_ctx* ctx, const float* fwd_fields, const pic_adj
       ctx->adj_tstart_len = need;
     }
   }
+  BucketCopies BC{};
   long long o = 0;
   for (int s = 0; s < ctx->ns; ++s) {
     AdjSpecies& S = AP.sp[s];
     S.tstart = nullptr;
     if (tiled && ctx->sp[s].n > 0) {
       int* t = ctx->d_adj_tstart + (long long)s * (nb + 1);
-      PIC_CK(ctx, cudaMemcpyAsync(t, sp[s].tstart, sizeof(int) * (nb + 1),
-                                  cudaMemcpyDeviceToDevice, ctx->st));
-      PIC_CK(ctx, launch_check_buckets(t, nb, ctx->sp[s].n, ctx->d_status, ctx->st, ctx->g.pdl));
+      BC.src[s] = sp[s].tstart;
+      BC.dst[s] = t;
+      BC.n[s] = ctx->sp[s].n;
       S.tstart = t;
     }
     S.dlist = ctx->d_dlist + o;
@@ -992,13 +1012,12 @@ pic_status pic_adjoint_step(pic_ctx* ctx, const float* fwd_fields, const pic_adj
     S.xbar = sp[s].xbar;
     S.ubar = sp[s].ubar;
   }
-  (void)D;
   const cudaError_t e = timed(ctx, PIC_KERNEL_ADJOINT, [&]() -> cudaError_t {
-    // forward fields seen by the particles: E and B1 = B - (c/2) curl+ E
-    cudaError_t r = cudaMemcpyAsync(ctx->d_adjF, fwd_fields, sizeof(float) * 6 * P,
-                                    cudaMemcpyDeviceToDevice, ctx->st);
-    if (r == cudaSuccess) r = launch_b_half(ctx->g, ctx->d_adjF, 0, ctx->st);
-    if (r == cudaSuccess) r = launch_adj_e(ctx->g, adj_fields, ctx->st);  // E' = E + c curl- B2 - Jf
+    // the bucket starts, checked; the forward fields seen by the particles, E and
+    // B1 = B - (c/2) curl+ E; and E' = E + c curl- B2 - Jf
+    cudaError_t r = adopt_buckets(ctx, BC);
+    if (r == cudaSuccess)
+      r = launch_adj_begin(ctx->g, fwd_fields, ctx->d_adjF, adj_fields, ctx->st);
     float* J = adj_fields + JX * P;
     float* a = J;
     float* b = ctx->d_jtmp;
@@ -1013,10 +1032,9 @@ pic_status pic_adjoint_step(pic_ctx* ctx, const float* fwd_fields, const pic_adj
     }
     if (r == cudaSuccess && a != J)
       r = cudaMemcpyAsync(J, a, sizeof(float) * 3 * P, cudaMemcpyDeviceToDevice, ctx->st);
-    if (r == cudaSuccess) r = launch_adj_b_half(ctx->g, adj_fields, ctx->st);  // B2 = B1 - ...
-    if (r == cudaSuccess) r = launch_adj_particles(AP, ctx->st);             // particles
-    if (r == cudaSuccess) r = launch_adj_b_half(ctx->g, adj_fields, ctx->st);  // B1 = B - ...
-    if (r == cudaSuccess) r = cudaMemsetAsync(J, 0, sizeof(float) * 3 * P, ctx->st);
+    if (r == cudaSuccess) r = launch_adj_b_half(ctx->g, adj_fields, 0, ctx->st);  // B2 = B1 - ...
+    if (r == cudaSuccess) r = launch_adj_particles(AP, ctx->st);                  // particles
+    if (r == cudaSuccess) r = launch_adj_b_half(ctx->g, adj_fields, 1, ctx->st);  // B1 = B - ...
     return r;
   });
   if (e != cudaSuccess) return cuda_fail(ctx, "adjoint step", e);
@@ -1061,20 +1079,23 @@ pic_status pic_sort_assume(pic_ctx* ctx, const int32_t* const* tstart) {
   for (int s = 0; s < ctx->ns; ++s)
     if (ctx->sp[s].n > 0 && !tstart[s])
       return set_err(ctx, PIC_ERR_ARG, "tstart of a species with particles is NULL");
-  const long long nb = sort_bins(ctx->tile);
+  // a tile kernel must never read a slot outside [0, n): starts that are not a
+  // partition are replaced by one bucket (correct, through the stray path) and
+  // reported by pic_check
+  BucketCopies BC{};
   for (int s = 0; s < ctx->ns; ++s) {
     const long long n = ctx->sp[s].n;
-    if (n > 0)
-      PIC_CK(ctx, cudaMemcpyAsync(ctx->d_tstart[s], tstart[s], sizeof(int) * (nb + 1),
-                                  cudaMemcpyDeviceToDevice, ctx->st));
-    else
-      PIC_CK(ctx, cudaMemsetAsync(ctx->d_tstart[s], 0, sizeof(int) * (nb + 1), ctx->st));
-    // a tile kernel must never read a slot outside [0, n): starts that are
-    // not a partition are replaced by one bucket (correct, through the stray
-    // path) and reported by pic_check
-    PIC_CK(ctx, launch_check_buckets(ctx->d_tstart[s], nb, n, ctx->d_status, ctx->st, ctx->g.pdl));
+    if (n > 0) {
+      BC.src[s] = tstart[s];
+      BC.dst[s] = ctx->d_tstart[s];
+      BC.n[s] = n;
+    } else {
+      PIC_CK(ctx, cudaMemsetAsync(ctx->d_tstart[s], 0,
+                                  sizeof(int) * (sort_bins(ctx->tile) + 1), ctx->st));
+    }
     ctx->sorted_n[s] = n;
   }
+  PIC_CK(ctx, adopt_buckets(ctx, BC));
   ctx->snapshot_valid = false;
   ctx->sorted_pending = false;
   ctx->sorted_step = ctx->steps;

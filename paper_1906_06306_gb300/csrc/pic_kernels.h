@@ -275,6 +275,15 @@ cudaError_t launch_clip_starts(const int* tstart, long long nb1, int lo, int hi,
                                cudaStream_t st);
 cudaError_t launch_check_buckets(int* tstart, long long nb, long long n, int* status,
                                  cudaStream_t st, int pdl);
+// dst[s] = src[s], checked in the same way, for every species with src[s], in
+// one launch; dcount[s] = 0
+struct BucketCopies {
+  const int* src[kMaxSpecies];
+  int* dst[kMaxSpecies];
+  long long n[kMaxSpecies];
+};
+cudaError_t launch_adopt_buckets(const BucketCopies& C, int nspecies, long long nb, int* dcount,
+                                 int* status, cudaStream_t st, int pdl);
 // out[r * ld + perm[i]] = in[r * ld + i] for i < n, r < rows (entries of perm
 // outside [0, n) skipped, ST_BAD_BUCKETS set)
 cudaError_t launch_unpermute(const int* perm, const float* in, float* out, long long n,
@@ -350,13 +359,15 @@ struct AdjParams {
   int* dcount;      // [nspecies] entries of the deferred lists
   AdjSpecies sp[kMaxSpecies];
 };
-// Bbar += c curl+ Ebar, Jbar = -Ebar (adjoint of the E update with -J)
-cudaError_t launch_adj_e(const GridDev& g, float* A, cudaStream_t st);
-// Ebar -= (c/2) curl- Bbar (adjoint of a B half step)
-cudaError_t launch_adj_b_half(const GridDev& g, float* A, cudaStream_t st);
+// F1 = (E, B - (c/2) curl+ E) of F; Bbar += c curl+ Ebar, Jbar = -Ebar (adjoint
+// of the E update with -J)
+cudaError_t launch_adj_begin(const GridDev& g, const float* F, float* F1, float* A,
+                             cudaStream_t st);
+// Ebar -= (c/2) curl- Bbar (adjoint of a B half step); with zero_j J = 0
+cudaError_t launch_adj_b_half(const GridDev& g, float* A, int zero_j, cudaStream_t st);
 // adjoint of gather + Boris + move + ZigZag for every particle: the tile pass
 // where every species gives its tile grouping (then the deferred ones through
-// global memory), else all through global memory
+// global memory; dcount is zero before), else all through global memory
 cudaError_t launch_adj_particles(const AdjParams& P, cudaStream_t st);
 
 }  // namespace pic

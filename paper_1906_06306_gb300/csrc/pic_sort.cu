@@ -449,8 +449,8 @@ cudaError_t launch_tile_scatter(const SortParams& P, const int* cell, const floa
 // 0 to n without decreasing; if not, every start but the last becomes 0 (one
 // bucket: the last tile's blocks take every particle, all through the stray
 // path) and the status word says so.
-__global__ void k_check_buckets(int* __restrict__ t, long long nb, long long n, int* status) {
-  grid_dependency();
+__device__ __forceinline__ void check_buckets(int* __restrict__ t, long long nb, long long n,
+                                              int* status) {
   bool bad = threadIdx.x == 0 && (t[0] != 0 || t[nb] != n);
   for (long long i = threadIdx.x; i < nb; i += blockDim.x) bad |= t[i] > t[i + 1];
   if (!__syncthreads_or(bad)) return;
@@ -461,10 +461,33 @@ __global__ void k_check_buckets(int* __restrict__ t, long long nb, long long n, 
   }
 }
 
+__global__ void k_check_buckets(int* __restrict__ t, long long nb, long long n, int* status) {
+  grid_dependency();
+  check_buckets(t, nb, n, status);
+}
+
 cudaError_t launch_check_buckets(int* tstart, long long nb, long long n, int* status,
                                  cudaStream_t st, int pdl) {
-  launch_kernel(pdl, k_check_buckets, 1, 1024, 0, st, tstart, nb, n, status);
-  return cudaGetLastError();
+  return launch_kernel(pdl, k_check_buckets, 1, 1024, 0, st, tstart, nb, n, status);
+}
+
+// Block s: species s's bucket starts, copied and checked.
+__global__ void __launch_bounds__(1024) k_adopt_buckets(const BucketCopies C, long long nb,
+                                                        int* dcount, int* status) {
+  grid_dependency();
+  const int s = blockIdx.x;
+  if (threadIdx.x == 0) dcount[s] = 0;
+  const int* src = C.src[s];
+  int* dst = C.dst[s];
+  if (!src) return;
+  for (long long i = threadIdx.x; i <= nb; i += blockDim.x) dst[i] = src[i];
+  __syncthreads();
+  check_buckets(dst, nb, C.n[s], status);
+}
+
+cudaError_t launch_adopt_buckets(const BucketCopies& C, int nspecies, long long nb, int* dcount,
+                                 int* status, cudaStream_t st, int pdl) {
+  return launch_kernel(pdl, k_adopt_buckets, nspecies, 1024, 0, st, C, nb, dcount, status);
 }
 
 // Bucket starts of one slot range [lo, hi) of a species: out[i] = tstart[i]

@@ -58,3 +58,35 @@ def test_chunks_with_more_bins_than_the_table_and_with_one(order):
     one = lambda rs, k: np.full(k, 12345)  # noqa: E731
     _run(2, shape, 600_000, many if order.startswith("random") else one, seed=3,
          tile=[2, 2] if order.startswith("random") else None)
+
+
+@pytest.mark.parametrize("tile", [[16, 16], [2, 2]])  # 2^13 bins: one launch; 2^16: a copy and a check each
+def test_adopted_bucket_starts_are_checked(tile):
+    import torch
+
+    from paper_1906_06306_gb300 import Simulation
+    from paper_1906_06306_gb300 import binding as B
+
+    rs = np.random.default_rng(5)
+    n = 5000
+    sp = [dict(q=q, m=1e-3, cell=rs.integers(0, 512 * 512, k).astype(np.int32),
+               off=rs.random((2, k), dtype=np.float32), u=np.zeros((3, k), np.float32))
+          for q, k in ((1e-3, n), (-1e-3, 0), (-1e-3, n - 1))]
+    sim = Simulation(2, 512, 512, 1, 0.45, np.zeros((9, 1, 512, 512), np.float32), sp,
+                     tuning=dict(tile=tile, sort_every=1000))
+    nb = B.pic_sort_bins(sim.ctx)
+    perm = [torch.empty(max(s["n"], 1), dtype=torch.int32, device=sim.device) for s in sim.species]
+    start = [torch.empty(nb + 1, dtype=torch.int32, device=sim.device) for _ in sim.species]
+    B.pic_sort_record(sim.ctx, [p.data_ptr() for p in perm], [t.data_ptr() for t in start])
+    B.pic_stats(sim.ctx)
+    B.pic_sort_assume(sim.ctx, [t.data_ptr() for t in start])
+    sim.step(2)
+    sim.check()
+    assert B.pic_stats(sim.ctx) == 0  # everyone in the window of its tile
+    bad = start[2].clone()
+    bad[nb // 2] = n + 7
+    B.pic_sort_assume(sim.ctx, [start[0].data_ptr(), start[1].data_ptr(), bad.data_ptr()])
+    with pytest.raises(B.PicError) as e:
+        sim.check()
+    assert e.value.status == B.PIC_ERR_STATE
+    sim.close()
