@@ -433,6 +433,11 @@ PushParams make_params(pic_ctx* ctx) {
   P.inv_c2 = 1.0f / (ctx->c * ctx->c);
   P.div0 = make_fastdiv(ctx->g.n[0]);
   P.div1 = make_fastdiv(ctx->g.n[1]);
+  P.div_splits = make_fastdiv(P.splits);
+  P.div_nt0 = make_fastdiv(P.t.nt[0]);
+  P.div_nt1 = make_fastdiv(P.t.nt[1]);
+  P.div_w0 = make_fastdiv(P.t.W[0]);
+  P.div_w1 = make_fastdiv(P.t.W[1]);
   P.wrap_fast = 1;
   for (int d = 0; d < ctx->grid.dim; ++d)
     if (ctx->g.n[d] < ctx->tile.W[d]) P.wrap_fast = 0;

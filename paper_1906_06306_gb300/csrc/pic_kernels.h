@@ -181,6 +181,8 @@ struct PushParams {
   int* status;
   float inv_c, inv_c2;
   FastDiv div0, div1;  // by n0 and n1: cell -> (i, j, k)
+  FastDiv div_splits, div_nt0, div_nt1;  // block -> tile -> its place
+  FastDiv div_w0, div_w1;                // window cell -> its place
   int wrap_fast;       // every axis has n >= window extent: one conditional wrap suffices
   float jq;            // quantum of the int32 shared-memory current (a power of 2)
   float jq_inv;        // 1 / jq

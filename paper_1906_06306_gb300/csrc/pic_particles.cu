@@ -435,10 +435,17 @@ __global__ void __launch_bounds__(kPushThreads, D == 3 ? PIC_PUSH_MIN_BLOCKS_3D
   __shared__ int q_n;      // entries in the stray queue (1D/2D)
   __shared__ int n_stray;  // particles of this block deferred as strays (3D)
   const GlobAcc GA{P.F, P.g.plane, P.g.n[0], P.g.n[1], P.g.n[2]};
-  const int tile = blockIdx.x / P.splits;
+  const int tile = fdiv(blockIdx.x, P.div_splits);
   const int split = blockIdx.x - tile * P.splits;
-  const int tc[3] = {tile % P.t.nt[0], (tile / P.t.nt[0]) % P.t.nt[1],
-                     tile / (P.t.nt[0] * P.t.nt[1])};
+  int tc[3] = {tile, 0, 0};
+  if (D >= 2) {
+    tc[1] = fdiv(tile, P.div_nt0);
+    tc[0] = tile - tc[1] * P.t.nt[0];
+  }
+  if (D == 3) {
+    tc[2] = fdiv(tc[1], P.div_nt1);
+    tc[1] -= tc[2] * P.t.nt[1];
+  }
   int w0[3] = {0, 0, 0};
 #pragma unroll
   for (int d = 0; d < D; ++d) w0[d] = tc[d] * P.t.T[d] - P.t.H;
@@ -469,13 +476,34 @@ __global__ void __launch_bounds__(kPushThreads, D == 3 ? PIC_PUSH_MIN_BLOCKS_3D
   const int lane = threadIdx.x & 31;
 
   float* ring = reinterpret_cast<float*>(queue + kQueueCap);  // TMA only
-  // the particles of this block: a contiguous share of each species' tile bucket
-  auto bucket = [&](int s, int& a, int& b) {
+  // The particles of this block, a contiguous share [a, b) of each species' tile
+  // bucket; shares differ by at most one particle.  (By every thread: bounds
+  // read from shared memory cost the 2D kernels 108 bytes of spills.)
+  const auto bucket = [&](int s, int& a, int& b) {
     const SpeciesDev& S = P.sp[s];
-    const long long lo = S.tstart[tile * P.t.nsub], hi = S.tstart[(tile + 1) * P.t.nsub];
-    const long long len = hi - lo;
-    a = (int)(lo + len * split / P.splits);
-    b = (int)(lo + len * (split + 1) / P.splits);
+    const int lo = S.tstart[tile * P.t.nsub], len = S.tstart[(tile + 1) * P.t.nsub] - lo;
+    const int q = fdiv(len, P.div_splits), r = len - q * P.splits;
+    a = lo + split * q + (split < r ? split : r);
+    b = a + q + (split < r ? 1 : 0);
+  };
+  // Window cell w: its place in the window, and in the lattice.
+  const auto place = [&](int w, int* l) {
+    if (FW0 > 0) {
+      l[0] = w % W0, l[1] = w / W0 % W1, l[2] = w / W0 / W1;
+    } else {
+      const int rr = D >= 2 ? fdiv(w, P.div_w0) : 0;
+      l[0] = w - rr * W0;
+      l[2] = D == 3 ? fdiv(rr, P.div_w1) : 0;
+      l[1] = rr - l[2] * W1;
+    }
+  };
+  const auto lattice = [&](const int* l) {  // a plane has fewer than 2^31 points
+    int x[3] = {w0[0] + l[0], D >= 2 ? w0[1] + l[1] : 0, D == 3 ? w0[2] + l[2] : 0};
+    if (!interior) {
+#pragma unroll
+      for (int d = 0; d < D; ++d) x[d] = P.wrap_fast ? wrap1(x[d], P.g.n[d]) : wrapi(x[d], P.g.n[d]);
+    }
+    return x[0] + P.g.n[0] * (x[1] + (D == 3 ? P.g.n[1] * x[2] : 0));
   };
   // producer state of the record stream (thread 0): species and first index of
   // the next batch to issue; pr_s == nspecies when everything is issued
@@ -555,8 +583,9 @@ __global__ void __launch_bounds__(kPushThreads, D == 3 ? PIC_PUSH_MIN_BLOCKS_3D
     }
   }
   for (int w = threadIdx.x; w < wc; w += blockDim.x) {
-    const int lx = w % W0, rr = w / W0, ly = rr % W1, lz = rr / W1;
-    const long long gi = GA.at(w0[0] + lx, w0[1] + ly, w0[2] + lz);
+    int l[3];
+    place(w, l);
+    const int lx = l[0], ly = l[1];
     if (MODE != 2) {
       float ex, ey, ez, bx, by, bz;
       if (win_tma) {  // box planes Ex .. Bz of box_x x box_y floats, x fastest
@@ -569,6 +598,7 @@ __global__ void __launch_bounds__(kPushThreads, D == 3 ? PIC_PUSH_MIN_BLOCKS_3D
         by = L[4 * pl];
         bz = L[5 * pl];
       } else {
+        const int gi = lattice(l);
         ex = __ldg(&P.F[EX * P.g.plane + gi]);
         ey = __ldg(&P.F[EY * P.g.plane + gi]);
         ez = __ldg(&P.F[EZ * P.g.plane + gi]);
@@ -639,9 +669,9 @@ __global__ void __launch_bounds__(kPushThreads, D == 3 ? PIC_PUSH_MIN_BLOCKS_3D
         for (int w = threadIdx.x; w < wc; w += blockDim.x) {
           const int v = ji[c * ws + w];
           if (v != 0) {
-            const int lx = w % W0, rr = w / W0, ly = rr % W1, lz = rr / W1;
-            const long long gi = GA.at(w0[0] + lx, w0[1] + ly, w0[2] + lz);
-            atomicAdd(&P.F[(JX + c) * P.g.plane + gi], (float)v * P.jq);
+            int l[3];
+            place(w, l);
+            atomicAdd(&P.F[(JX + c) * P.g.plane + lattice(l)], (float)v * P.jq);
             ji[c * ws + w] = 0;
           }
         }
@@ -821,8 +851,9 @@ __global__ void __launch_bounds__(kPushThreads, D == 3 ? PIC_PUSH_MIN_BLOCKS_3D
     spill();
     __syncthreads();
     for (int w = threadIdx.x; w < (kFoldGlobal<D> ? 0 : wc); w += blockDim.x) {
-      const int lx = w % W0, rr = w / W0, ly = rr % W1, lz = rr / W1;
-      const long long gi = GA.at(w0[0] + lx, w0[1] + ly, w0[2] + lz);
+      int l[3];
+      place(w, l);
+      const int gi = lattice(l);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         const float v = jf[c * ws + w];
