@@ -445,6 +445,14 @@ PushParams make_params(pic_ctx* ctx) {
   for (int s = 0; s < ctx->ns; ++s) maxq = std::fmax(maxq, std::fabs(ctx->sp[s].q));
   P.jq = current_quantum(maxq, ctx->c, kPushThreads * kSpillEvery);
   P.jq_inv = 1.0f / P.jq;
+  // the most batches with 1.25 c batch max|q| < 2^31 quanta (see current_quantum)
+  const double per_batch = 1.25 * (double)ctx->c * kPushThreads * (double)maxq;
+  P.spill_every = kSpillEvery;
+  while (P.spill_every < 2 * kSpillEvery &&
+         per_batch * (P.spill_every + 1) < std::ldexp((double)P.jq, 31))
+    ++P.spill_every;
+  P.quads = ctx->g.n[0] % 4 == 0 && ctx->g.plane % 4 == 0 &&
+            (reinterpret_cast<uintptr_t>(ctx->F) & 15) == 0;
   long long o = 0;
   for (int s = 0; s < ctx->ns; ++s) {
     SpeciesDev& S = P.sp[s];

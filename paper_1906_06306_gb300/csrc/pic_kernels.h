@@ -121,12 +121,15 @@ constexpr int kSubTile3[3] = {PIC_SUBTILE3_X, PIC_SUBTILE3_Y, PIC_SUBTILE3_Z};
 // Sort bins of a tiling: sub-tiles of every tile, tile-major.
 inline long long sort_bins(const TileDev& t) { return (long long)t.ntiles * t.nsub; }
 constexpr int kPushThreads = PIC_PUSH_THREADS;
-constexpr int kSpillEvery = PIC_SPILL_EVERY;  // batches of kPushThreads particles between spills
+// Batches of kPushThreads particles that the current's quantum is chosen for; a
+// launch folds after as many more as that quantum still has room for (up to
+// twice as many: a power of 2 is rounded up to), so that most blocks fold once.
+constexpr int kSpillEvery = PIC_SPILL_EVERY;
 // Shared-memory queue of the 1D/2D tile kernels for particles outside the tile
 // window (about 0.5 % of the particles between sorts).  It is drained at the
 // end of each species and at a spill point where it is more than half full; a
 // stray that finds it full is processed at once by its own lane.
-constexpr int kQueueCap = 512;
+constexpr int kQueueCap = 1024;
 // Particle records of a batch streamed into shared memory by bulk copies
 // (1D/2D fused kernels): a ring of this many stages of kPushThreads records.
 constexpr int kRecStages = 2;
@@ -186,6 +189,8 @@ struct PushParams {
   int wrap_fast;       // every axis has n >= window extent: one conditional wrap suffices
   float jq;            // quantum of the int32 shared-memory current (a power of 2)
   float jq_inv;        // 1 / jq
+  int spill_every;     // batches between folds of the int32 current
+  int quads;           // J's rows are whole aligned quads of x points
   unsigned long long* strays;  // running count of particles that took the global path
   int pusher;                  // 0 Boris (Appendix C), 1 Higuera-Cary
   int wall;                    // conducting wall on the node plane x = wall (0: none)

@@ -13,7 +13,7 @@
 //   then int32 Jx Jy Jz (fixed point) and float Jx Jy Jz (running sums).
 // Components that share a stencil share their loads.  The current goes into
 // the int32 window with native integer atomics (same-address lanes do not
-// serialise) and is folded into the float window after every kSpillEvery
+// serialise) and is folded into the float window after every spill_every
 // batches of blockDim particles, before any int32 word can overflow.
 //
 // A particle whose stencil is not inside the window (it drifted more than
@@ -661,21 +661,53 @@ __global__ void __launch_bounds__(kPushThreads, D == 3 ? PIC_PUSH_MIN_BLOCKS_3D
   }
   __syncthreads();
 
+  // Add the window's current to the lattice's J planes; take(c, w) is component
+  // c's sum at window cell w.  Where rows are whole aligned quads of x points,
+  // a quad goes by one vector reduction (zeros outside the window): the L2's
+  // atomic units take one reduction at a time, word or quad, and 3D windows
+  // with their halos add some 2000 words a block.  (1D windows are too small:
+  // word by word more threads take part.)
+  const auto add_to_lattice = [&](auto take) {
+    float* J = P.F + JX * P.g.plane;
+    if (D > 1 && P.quads) {
+      const int lead = w0[0] & 3, nq = (lead + W0 + 3) >> 2, rows = wc / W0;
+      for (int t = threadIdx.x; t < nq * rows; t += blockDim.x) {
+        const int r = t / nq, x = 4 * (t - r * nq) - lead;
+        const int l[3] = {x, D == 3 ? r % W1 : r, D == 3 ? r / W1 : 0};
+        float* to = J + lattice(l);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          float v[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            v[e] = (unsigned)(x + e) < (unsigned)W0 ? take(c, r * W0 + x + e) : 0.f;
+          if (v[0] != 0.f || v[1] != 0.f || v[2] != 0.f || v[3] != 0.f)
+            atomicAdd(reinterpret_cast<float4*>(to + c * P.g.plane),
+                      make_float4(v[0], v[1], v[2], v[3]));
+        }
+      }
+      return;
+    }
+    for (int w = threadIdx.x; w < wc; w += blockDim.x) {
+      int l[3];
+      place(w, l);
+      float* to = J + lattice(l);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const float v = take(c, w);
+        if (v != 0.f) atomicAdd(to + c * P.g.plane, v);
+      }
+    }
+  };
   // between barriers: fold the int32 window into the float window, clear it
   auto spill = [&]() {
     if constexpr (kFoldGlobal<D>) {
       // the fixed-point sums go straight to the global J planes, then are cleared
-      for (int c = 0; c < 3; ++c) {
-        for (int w = threadIdx.x; w < wc; w += blockDim.x) {
-          const int v = ji[c * ws + w];
-          if (v != 0) {
-            int l[3];
-            place(w, l);
-            atomicAdd(&P.F[(JX + c) * P.g.plane + lattice(l)], (float)v * P.jq);
-            ji[c * ws + w] = 0;
-          }
-        }
-      }
+      add_to_lattice([&](int c, int w) {
+        const int v = ji[c * ws + w];
+        if (v != 0) ji[c * ws + w] = 0;
+        return (float)v * P.jq;
+      });
       return;
     }
     if constexpr (kJ64<D>) {
@@ -733,7 +765,7 @@ __global__ void __launch_bounds__(kPushThreads, D == 3 ? PIC_PUSH_MIN_BLOCKS_3D
   };
 
   // Particles kPushThreads at a time (with PIC_PREFETCH the record of the next
-  // batch is loaded while the current one is processed).  Every kSpillEvery
+  // batch is loaded while the current one is processed).  Every spill_every
   // batches (and only there) the block synchronises, folds the current and, in
   // 1D/2D, drains the stray queue if it could overflow in the next round.
   int batches = 0;
@@ -822,7 +854,7 @@ __global__ void __launch_bounds__(kPushThreads, D == 3 ? PIC_PUSH_MIN_BLOCKS_3D
         }
       }
       if (PIC_PREFETCH) cur = nxt;
-      if (++batches == kSpillEvery) {
+      if (++batches == P.spill_every) {
         batches = 0;
         __syncthreads();
         const int qn = q_n;  // read by every thread before anyone can queue again
@@ -850,16 +882,8 @@ __global__ void __launch_bounds__(kPushThreads, D == 3 ? PIC_PUSH_MIN_BLOCKS_3D
   if (MODE != 1) {
     spill();
     __syncthreads();
-    for (int w = threadIdx.x; w < (kFoldGlobal<D> ? 0 : wc); w += blockDim.x) {
-      int l[3];
-      place(w, l);
-      const int gi = lattice(l);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const float v = jf[c * ws + w];
-        if (v != 0.0f) atomicAdd(&P.F[(JX + c) * P.g.plane + gi], v);
-      }
-    }
+    if constexpr (!kFoldGlobal<D>)
+      add_to_lattice([&](int c, int w) { return jf[c * ws + w]; });
   }
 }
 
