@@ -451,15 +451,28 @@ template <int D>
 __device__ __forceinline__ AdjBlock adj_block(const AdjParams& P) {
   const TileDev& t = P.t;
   AdjBlock B;
-  B.tile = blockIdx.x / P.splits;
-  B.split = blockIdx.x % P.splits;
-  const int tc[3] = {B.tile % t.nt[0], (B.tile / t.nt[0]) % t.nt[1], B.tile / (t.nt[0] * t.nt[1])};
+  B.tile = fdiv((int)blockIdx.x, P.div_splits);
+  B.split = (int)blockIdx.x - B.tile * P.splits;
+  const int r = fdiv(B.tile, P.div_nt0), z = fdiv(r, P.div_nt1);
+  const int tc[3] = {B.tile - r * t.nt[0], r - z * t.nt[1], z};
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     B.w0[d] = d < D ? tc[d] * t.T[d] - t.H : 0;
     B.W[d] = d < D ? t.W[d] : 1;
   }
   return B;
+}
+// The lattice point of the window's place l, as an index into a plane (fewer
+// than 2^31 points).
+template <int D>
+__device__ __forceinline__ int adj_lattice(const AdjParams& P, const AdjBlock& B, const int* l) {
+  int x[3] = {0, 0, 0};
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    const int i = B.w0[d] + l[d];
+    x[d] = P.wrap_fast ? wrap1(i, P.g.n[d]) : wrapi(i, P.g.n[d]);
+  }
+  return x[0] + P.g.n[0] * (x[1] + (D == 3 ? P.g.n[1] * x[2] : 0));
 }
 // Window-local cell of a particle and whether its stencil (cells b - 1 ..
 // b + 2 on every gridded axis, as in the forward tile kernel) is inside the
@@ -473,17 +486,37 @@ __device__ __forceinline__ bool adj_in_window(const AdjParams& P, const AdjBlock
   l[0] = l[1] = l[2] = 0;
 #pragma unroll
   for (int d = 0; d < D; ++d) {
-    l[d] = wrapi(ijk[d] - B.w0[d], P.g.n[d]);
+    // a cell is in [0, n) and a window starts in [-H, n): one conditional wrap
+    // where no axis is shorter than the window (and so than H)
+    const int i = ijk[d] - B.w0[d];
+    l[d] = P.wrap_fast ? wrap1(i, P.g.n[d]) : wrapi(i, P.g.n[d]);
     inwin &= (unsigned)(l[d] - 1) <= (unsigned)(B.W[d] - 4);
   }
   return inwin;
 }
-// This block's share [a, b) of species s's tile bucket.
+// This block's share [a, b) of species s's tile bucket; shares differ by at most
+// one particle.
 __device__ __forceinline__ void adj_share(const AdjParams& P, const AdjSpecies& S,
-                                          const AdjBlock& B, long long& a, long long& b) {
-  const long long lo = S.tstart[B.tile * P.t.nsub], hi = S.tstart[(B.tile + 1) * P.t.nsub];
-  a = lo + (hi - lo) * B.split / P.splits;
-  b = lo + (hi - lo) * (B.split + 1) / P.splits;
+                                          const AdjBlock& B, int& a, int& b) {
+  const int lo = S.tstart[B.tile * P.t.nsub], len = S.tstart[(B.tile + 1) * P.t.nsub] - lo;
+  const int q = fdiv(len, P.div_splits), r = len - q * P.splits;
+  a = lo + B.split * q + (B.split < r ? B.split : r);
+  b = a + q + (B.split < r ? 1 : 0);
+}
+// q = 2^(e - 22) and 1/q for M < 2^e, M's exponent from frexpf: where q and 1/q
+// are normal numbers they are put together from M's exponent bits (frexpf and
+// two ldexpf took some 40 instructions of a batch).
+__device__ __forceinline__ void adj_quantum(unsigned mb, float& q, float& inv_q) {
+  const unsigned ef = mb >> 23;  // e + 126
+  if (ef >= 22 && ef < 255) {
+    q = __uint_as_float((ef - 21) << 23);
+    inv_q = __uint_as_float((275 - ef) << 23);
+  } else {
+    int e = 0;
+    frexpf(__uint_as_float(mb), &e);
+    q = ldexpf(1.0f, e - 22);
+    inv_q = ldexpf(1.0f, 22 - e);
+  }
 }
 
 // The tile pass (particles grouped by tile): one block per (tile, split)
@@ -499,6 +532,12 @@ __device__ __forceinline__ void adj_share(const AdjParams& P, const AdjSpecies& 
 // 2^30; after every batch the integers are folded into an FP32 window, which
 // goes to the lattice once per window cell.  A particle whose stencil is not
 // inside the window goes on the species' deferred list for the global pass.
+// Bound by instruction issue and by the latency of the reverse chain (64
+// registers, 4 blocks an SM), so what is not the chain is kept small: places
+// and shares by multiply-shift, conditional wraps, the quantum from exponent
+// bits, two barriers a batch, quads to the lattice.  With 64-bit divisions,
+// remainders, frexpf/ldexpf, a third barrier and single words a launch of
+// 128^2 cells x 64 particles took 74.1 us, so it takes 57.4.
 template <int D>
 __global__ void __launch_bounds__(256, D == 3 ? 2 : PIC_ADJ_MIN_BLOCKS)
     k_adj_tiles(const AdjParams P) {
@@ -508,21 +547,25 @@ __global__ void __launch_bounds__(256, D == 3 ? 2 : PIC_ADJ_MIN_BLOCKS)
   const AdjBlock B = adj_block<D>(P);
   const int wc = P.t.wcells, ws = P.t.wstride;
   const long long plane = P.g.plane;
-  const GlobAcc G{P.A, plane, P.g.n[0], P.g.n[1], P.g.n[2]};
   int* wi = reinterpret_cast<int*>(sm + 9 * ws);  // 6 planes of fixed-point sums
   float* wf = sm + 15 * ws;                       // 6 planes of their FP32 folds
+  const auto place = [&](int w, int* l) {  // window cell w's place in the window
+    const int rr = D >= 2 ? fdiv(w, P.div_w0) : 0;
+    l[0] = w - rr * B.W[0];
+    l[2] = D == 3 ? fdiv(rr, P.div_w1) : 0;
+    l[1] = rr - l[2] * B.W[1];
+  };
   for (int w = threadIdx.x; w < wc; w += blockDim.x) {
-    const int lx = w % B.W[0], rr = w / B.W[0], ly = rr % B.W[1], lz = rr / B.W[1];
-    const long long gi = G.at(B.w0[0] + lx, B.w0[1] + ly, B.w0[2] + lz);
+    int l[3];
+    place(w, l);
+    const int gi = adj_lattice<D>(P, B, l);
 #pragma unroll
     for (int c = 0; c < 6; ++c) sm[c * ws + w] = __ldg(&P.F1[c * plane + gi]);
 #pragma unroll
     for (int a = 0; a < 3; ++a) sm[(6 + a) * ws + w] = P.A[(JX + a) * plane + gi];
   }
-  for (int w = threadIdx.x; w < 6 * ws; w += blockDim.x) {
-    wi[w] = 0;
-    wf[w] = 0.f;
-  }
+  for (int w = threadIdx.x; w < 12 * ws / 4; w += blockDim.x)
+    reinterpret_cast<int4*>(wi)[w] = make_int4(0, 0, 0, 0);
   __syncthreads();
   const AdjWin WN{sm, B.W[0], B.W[0] * B.W[1], ws};
   const int W0 = B.W[0], W01 = B.W[0] * B.W[1];
@@ -530,11 +573,11 @@ __global__ void __launch_bounds__(256, D == 3 ? 2 : PIC_ADJ_MIN_BLOCKS)
   for (int s = 0; s < P.nspecies; ++s) {
     const AdjSpecies& S = P.sp[s];
     if (S.n == 0) continue;
-    long long a, b;
+    int a, b;
     adj_share(P, S, B, a, b);
     const long long ld = S.ld;
-    for (long long base = a; base < b; base += blockDim.x) {  // the same count for every thread
-      const long long p = base + threadIdx.x;
+    for (int base = a; base < b; base += blockDim.x) {  // the same count for every thread
+      const int p = base + threadIdx.x;
       float ebb[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, o[3] = {0.f, 0.f, 0.f}, xb[3];
       int l[3] = {0, 0, 0};
       bool mine = false;
@@ -545,7 +588,7 @@ __global__ void __launch_bounds__(256, D == 3 ? 2 : PIC_ADJ_MIN_BLOCKS)
             adj_chain<D>(WN, WN, S, p, l, c, o, xb, ebb);
             mine = true;
           } else {
-            S.dlist[atomicAdd(&P.dcount[s], 1)] = (int)p;
+            S.dlist[atomicAdd(&P.dcount[s], 1)] = p;
           }
         }
       }
@@ -559,10 +602,8 @@ __global__ void __launch_bounds__(256, D == 3 ? 2 : PIC_ADJ_MIN_BLOCKS)
       unsigned mb = 0u;
 #pragma unroll
       for (int k = 0; k < 8; ++k) mb = max(mb, wmax[k]);
-      const float M = __uint_as_float(mb);
-      int e = 0;
-      frexpf(M, &e);  // M < 2^e
-      const float q = ldexpf(1.0f, e - 22), inv_q = ldexpf(1.0f, 22 - e);
+      float q, inv_q;
+      adj_quantum(mb, q, inv_q);
       if (mine) {
         // the gather's reverse (gather_adj's operations, in its order, for the
         // position gradient) with each term also added, in quanta, to the window
@@ -621,12 +662,37 @@ __global__ void __launch_bounds__(256, D == 3 ? 2 : PIC_ADJ_MIN_BLOCKS)
           }
         }
       }
-      __syncthreads();
+      // no barrier here: the integers are next added to after the next batch's
+      // first one, so the fold overlaps other warps' reverse chain
     }
   }
+  __syncthreads();
+  if (D > 1 && P.quads) {
+    // rows are whole aligned quads of x points: a quad goes by one vector
+    // reduction (zeros outside the window), as the L2's atomic units take one
+    // reduction at a time, word or quad
+    const int W0r = B.W[0], lead = B.w0[0] & 3, nq = (lead + W0r + 3) >> 2, rows = wc / W0r;
+    for (int t = threadIdx.x; t < nq * rows; t += blockDim.x) {
+      const int r = t / nq, x = 4 * (t - r * nq) - lead, z = D == 3 ? fdiv(r, P.div_w1) : 0;
+      const int l[3] = {x, r - z * B.W[1], z};
+      float* to = P.A + adj_lattice<D>(P, B, l);
+#pragma unroll
+      for (int c2 = 0; c2 < 6; ++c2) {
+        float v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          v[k] = (unsigned)(x + k) < (unsigned)W0r ? wf[c2 * ws + r * W0r + x + k] : 0.f;
+        if (v[0] != 0.f || v[1] != 0.f || v[2] != 0.f || v[3] != 0.f)
+          atomicAdd(reinterpret_cast<float4*>(to + c2 * plane),
+                    make_float4(v[0], v[1], v[2], v[3]));
+      }
+    }
+    return;
+  }
   for (int w = threadIdx.x; w < wc; w += blockDim.x) {
-    const int lx = w % B.W[0], rr = w / B.W[0], ly = rr % B.W[1], lz = rr / B.W[1];
-    const long long gi = G.at(B.w0[0] + lx, B.w0[1] + ly, B.w0[2] + lz);
+    int l[3];
+    place(w, l);
+    const int gi = adj_lattice<D>(P, B, l);
 #pragma unroll
     for (int c2 = 0; c2 < 6; ++c2) {
       const float v = wf[c2 * ws + w];

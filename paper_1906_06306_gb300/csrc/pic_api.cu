@@ -985,6 +985,16 @@ pic_status pic_adjoint_step(pic_ctx* ctx, const float* fwd_fields, const pic_adj
   AP.A = adj_fields;
   AP.div0 = make_fastdiv(ctx->g.n[0]);
   AP.div1 = make_fastdiv(ctx->g.n[1]);
+  AP.div_splits = make_fastdiv(AP.splits);
+  AP.div_nt0 = make_fastdiv(AP.t.nt[0]);
+  AP.div_nt1 = make_fastdiv(AP.t.nt[1]);
+  AP.div_w0 = make_fastdiv(AP.t.W[0]);
+  AP.div_w1 = make_fastdiv(AP.t.W[1]);
+  AP.wrap_fast = 1;
+  for (int d = 0; d < ctx->grid.dim; ++d)
+    if (ctx->g.n[d] < AP.t.W[d]) AP.wrap_fast = 0;
+  AP.quads = ctx->g.n[0] % 4 == 0 && P % 4 == 0 &&
+             (reinterpret_cast<uintptr_t>(adj_fields) & 15) == 0;
   AP.nspecies = ctx->ns;
   AP.dcount = ctx->d_dcount;
   // the tile grouping: the caller's bucket starts, copied and checked (a tile

@@ -362,6 +362,9 @@ struct AdjParams {
   const float* F1;  // forward E and the B of the first half step (9-plane layout)
   float* A;         // adjoint planes: Ebar, Bbar, Jbar
   FastDiv div0, div1;  // by n0 and n1: cell -> (i, j, k)
+  FastDiv div_splits, div_nt0, div_nt1, div_w0, div_w1;  // block -> tile, window cell -> place
+  int wrap_fast;       // every axis has n >= window extent: one conditional wrap suffices
+  int quads;           // the rows of A's planes are whole 16-byte quads
   int nspecies;
   int* dcount;      // [nspecies] entries of the deferred lists
   AdjSpecies sp[kMaxSpecies];
