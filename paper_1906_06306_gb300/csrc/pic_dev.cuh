@@ -161,13 +161,13 @@ struct SpeciesDev {
 // less than 1, so x M / 2^s exceeds x / d by less than x / 2^s < 2^-l <= 1/d,
 // which cannot carry the fractional part of x / d (at most 1 - 1/d) past 1.
 struct FastDiv {
-  unsigned long long M;
+  unsigned M;
   int s;
   int d;
 };
 
 __device__ __forceinline__ int fdiv(int x, const FastDiv& f) {
-  return (int)(((unsigned long long)(unsigned)x * f.M) >> f.s);
+  return (int)(((unsigned long long)(unsigned)x * f.M) >> f.s);  // 32 x 32 -> 64 bits
 }
 
 __device__ __forceinline__ int wrapi(int i, int n) {

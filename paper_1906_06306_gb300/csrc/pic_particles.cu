@@ -960,7 +960,7 @@ FastDiv make_fastdiv(int d) {
   const int s = 31 + l;
   const unsigned long long two_s = 1ULL << s;
   FastDiv f;
-  f.M = (two_s + (unsigned long long)d - 1) / (unsigned long long)d;
+  f.M = (unsigned)((two_s + (unsigned long long)d - 1) / (unsigned long long)d);
   f.s = s;
   f.d = d;
   return f;

@@ -27,11 +27,12 @@ __global__ void k_wall_fields(float* __restrict__ F, const GridDev g, int w, int
   const int n0 = g.n[0];
   const long long P = g.plane;
   const int cols = w + 1 + (n0 - i_zero);
-  const long long rows = P / n0;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < rows * cols;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int col = (int)(idx % cols);
-    const long long row = (idx / cols) * n0;
+  const unsigned work = (unsigned)(P / n0) * cols;  // at most a plane's points, fewer than 2^31
+  for (unsigned idx = blockIdx.x * blockDim.x + threadIdx.x; idx < work;
+       idx += gridDim.x * blockDim.x) {
+    const unsigned r = idx / (unsigned)cols;
+    const int col = (int)(idx - r * cols);
+    const long long row = (long long)r * n0;
     if (col < w) {
       const long long a = row + col, ri = row + (2 * w - col), rh = row + (2 * w - 1 - col);
       F[EX * P + a] = F[EX * P + rh];
