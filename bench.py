@@ -135,6 +135,14 @@ def fused_away(sim):
     return 0 if passes < 2 else passes - 2 * -(-passes // (2 * most))
 
 
+def sort_shared(sim):
+    """Launches of launches_per_step's sort that the species share: all of them
+    take one count, one scan and one scatter."""
+    from paper_1906_06306_gb300 import binding as B
+
+    return (3 if B.pic_sort_bins(sim.ctx) <= 4096 else 5) * (sim.nspecies - 1)
+
+
 def profiled_traffic(workload, full_size, nparticles):
     """DRAM bytes per launch of the fused particle kernel from the workload's
     committed ncu summary, if it was taken on the current kernel source: the
@@ -892,6 +900,7 @@ def run_ours(args):
     nsorts = -(-args.steps // tun["sort_every"])  # at most one sort per cadence in the loop
     per_step, per_sort = launches_per_step(sim, shock)
     per_step -= fused_away(sim)
+    per_sort -= sort_shared(sim)
     launches = args.steps * per_step + nsorts * per_sort
     if shock:  # per step: 3 wall-field passes, the injection, and the tail kernel on
         # every step that does not start with a sort

@@ -46,8 +46,8 @@ struct pic_ctx {
   bool ensemble = false;  // being captured into a batch graph
   long long ntot = 0, nmax = 0;
   int* d_tstart[PIC_MAX_SPECIES] = {};
-  int* d_count = nullptr;   // per tile
-  int* d_cursor = nullptr;  // per tile
+  int* d_count = nullptr;   // per species and tile
+  int* d_cursor = nullptr;  // per species and tile
   void* d_sortbuf = nullptr;   // sorted particles of every species (one record layout each)
   bool sorted_pending = false;  // the next push reads the sorted buffer (no copy back)
   int* d_cell_old = nullptr;
@@ -303,9 +303,10 @@ pic_status alloc_tiles(pic_ctx* ctx) {
   }
   dfree(ctx->d_count);
   dfree(ctx->d_cursor);
-  // the counts, then the multi-block scan's scratch
-  PIC_CK(ctx, dalloc(&ctx->d_count, sort_bins(ctx->tile) + scan_scratch(sort_bins(ctx->tile))));
-  PIC_CK(ctx, dalloc(&ctx->d_cursor, sort_bins(ctx->tile)));
+  // per species the counts, then the multi-block scan's scratch
+  const long long bins = sort_bins(ctx->tile);
+  PIC_CK(ctx, dalloc(&ctx->d_count, ctx->ns * (bins + scan_scratch(bins))));
+  PIC_CK(ctx, dalloc(&ctx->d_cursor, ctx->ns * bins));
   window_map(ctx);
   return PIC_OK;
 }
@@ -497,37 +498,48 @@ PushParams make_params(pic_ctx* ctx) {
   return P;
 }
 
-// Sort every species by tile into the sorted buffer.  With copy_back the
-// sorted particles are copied into the caller's arrays; without, the next push
-// reads them from the buffer and writes the caller's arrays (pic_step).
-// The launches that sort species s by tile into its part of the sorted
-// buffer (and, with copy_back, copy it back into the caller's arrays).
-cudaError_t sort_species(pic_ctx* ctx, int s, bool copy_back, int32_t* perm) {
+// Sort species s0 .. s1 - 1 by tile into the sorted buffer, in launches that
+// they share.  With copy_back the sorted particles are copied into the caller's
+// arrays; without, the next push reads them from the buffer and writes the
+// caller's arrays (pic_step).
+cudaError_t sort_species(pic_ctx* ctx, int s0, int s1, bool copy_back, int32_t* const* perm) {
   const SortParams P = make_sort_params(ctx->g, ctx->tile, ctx->d_status);
   const int D = ctx->grid.dim;
-  const long long n = ctx->sp[s].n, ld = ctx->cap[s];
-  const int bins = (int)sort_bins(ctx->tile);
-  cudaError_t r = cudaMemsetAsync(ctx->d_count, 0, sizeof(int) * bins, ctx->st);
-  if (r != cudaSuccess) return r;
-  r = launch_tile_count(P, ctx->sp[s].cell, n, ctx->d_count, ctx->st);
-  if (r != cudaSuccess) return r;
-  r = launch_tile_scan(ctx->d_count, bins, ctx->d_tstart[s], ctx->d_cursor, ctx->d_count + bins,
-                       ctx->st, ctx->g.pdl);
-  if (r != cudaSuccess) return r;
-  if (n == 0) return cudaSuccess;
-  int* cell_out = (int*)ctx->d_sortbuf + sortbuf_offset(ctx, s);
-  float* off_out = (float*)(cell_out + ld);
-  float* u_out = off_out + (long long)D * ld;
-  r = launch_tile_scatter(P, ctx->sp[s].cell, ctx->sp[s].off, ctx->sp[s].u, n, ld, ctx->d_cursor,
-                          cell_out, off_out, u_out, ctx->st, perm);
-  if (r != cudaSuccess) return r;
-  if (!copy_back) return cudaSuccess;
+  const long long bins = sort_bins(ctx->tile), stride = bins + scan_scratch(bins);
+  SortSet Q{};
+  for (int s = s0; s < s1; ++s) {
+    SortSpecies& S = Q.sp[Q.ns++];
+    S.cell = ctx->sp[s].cell;
+    S.off = ctx->sp[s].off;
+    S.u = ctx->sp[s].u;
+    S.n = ctx->sp[s].n;
+    S.ld = ctx->cap[s];
+    S.count = ctx->d_count + s * stride;
+    S.scratch = S.count + bins;
+    S.start = ctx->d_tstart[s];
+    S.cursor = ctx->d_cursor + s * bins;
+    S.cell_out = (int*)ctx->d_sortbuf + sortbuf_offset(ctx, s);
+    S.off_out = (float*)(S.cell_out + S.ld);
+    S.u_out = S.off_out + (long long)D * S.ld;
+    S.perm = perm ? perm[s] : nullptr;
+  }
+  cudaError_t r = cudaMemsetAsync(Q.sp[0].count, 0, sizeof(int) * stride * Q.ns, ctx->st);
+  if (r == cudaSuccess) r = launch_tile_count(P, Q, ctx->st);
+  if (r == cudaSuccess) r = launch_tile_scan(Q, (int)bins, ctx->st, ctx->g.pdl);
+  if (r == cudaSuccess) r = launch_tile_scatter(P, Q, ctx->st);
+  if (r != cudaSuccess || !copy_back) return r;
   const cudaMemcpyKind k = cudaMemcpyDeviceToDevice;
-  r = copy_rows(ctx->sp[s].cell, cell_out, sizeof(int), n, ld, 1, k, ctx->st);
-  if (r != cudaSuccess) return r;
-  r = copy_rows(ctx->sp[s].off, off_out, sizeof(float), n, ld, D, k, ctx->st);
-  if (r != cudaSuccess) return r;
-  return copy_rows(ctx->sp[s].u, u_out, sizeof(float), n, ld, 3, k, ctx->st);
+  for (int s = s0; s < s1; ++s) {
+    const SortSpecies& S = Q.sp[s - s0];
+    if (S.n == 0) continue;
+    r = copy_rows(ctx->sp[s].cell, S.cell_out, sizeof(int), S.n, S.ld, 1, k, ctx->st);
+    if (r != cudaSuccess) return r;
+    r = copy_rows(ctx->sp[s].off, S.off_out, sizeof(float), S.n, S.ld, D, k, ctx->st);
+    if (r != cudaSuccess) return r;
+    r = copy_rows(ctx->sp[s].u, S.u_out, sizeof(float), S.n, S.ld, 3, k, ctx->st);
+    if (r != cudaSuccess) return r;
+  }
+  return cudaSuccess;
 }
 
 // Bucket starts handed in from outside, copied and checked (every species with
@@ -574,11 +586,7 @@ void sort_done(pic_ctx* ctx, bool copy_back) {
 
 pic_status do_sort(pic_ctx* ctx, bool copy_back, int32_t* const* perm = nullptr) {
   const cudaError_t e = timed(ctx, PIC_KERNEL_SORT, [&]() -> cudaError_t {
-    for (int s = 0; s < ctx->ns; ++s) {
-      const cudaError_t r = sort_species(ctx, s, copy_back, perm ? perm[s] : nullptr);
-      if (r != cudaSuccess) return r;
-    }
-    return cudaSuccess;
+    return sort_species(ctx, 0, ctx->ns, copy_back, perm);
   });
   if (e != cudaSuccess) return cuda_fail(ctx, "tile sort", e);
   sort_done(ctx, copy_back);
@@ -1487,7 +1495,7 @@ pic_status step_host_copies(pic_ctx* ctx, const pic_host_species* hs, float* hos
   for (int s = 0; s < ns; ++s) {
     if (sort) {  // the count covers the whole species
       PIC_CK(ctx, cudaStreamWaitEvent(ctx->st, ev_in(s, nk[s] - 1), 0));
-      if ((e = sort_species(ctx, s, false, nullptr)) != cudaSuccess)
+      if ((e = sort_species(ctx, s, s + 1, false, nullptr)) != cudaSuccess)
         return cuda_fail(ctx, "tile sort", e);
     }
     for (int k = 0; k < nk[s]; ++k) {

@@ -261,20 +261,34 @@ struct SortParams {
   FastDiv dt0, dt1, dt2;     // by the tile extents: lattice point -> tile
   FastDiv ds0, ds1, ds2;     // by the sub-tile extents: tile-local point -> sub-tile
 };
+// One species' part of a sort: particle arrays with rows of ld elements, the
+// first n of which are particles, and where they go
+struct SortSpecies {
+  const int* cell;
+  const float* off;
+  const float* u;
+  long long n, ld;
+  int* count;    // [bins], cleared before the count
+  int* start;    // [bins + 1] bucket starts
+  int* cursor;   // [bins]
+  int* scratch;  // [scan_scratch(bins)]
+  int* cell_out;
+  float* off_out;
+  float* u_out;
+  int* perm;     // or null: perm[new slot] = old slot
+};
+// The species that share a sort's launches (blockIdx.y, or the scan's blocks)
+struct SortSet {
+  int ns;
+  SortSpecies sp[kMaxSpecies];
+};
 SortParams make_sort_params(const GridDev& g, const TileDev& t, int* status);
-cudaError_t launch_tile_count(const SortParams& P, const int* cell, long long n, int* count,
-                              cudaStream_t st);
-// exclusive scan of count[0..n) into start[0..n] and cursor; n above 4096 uses
-// scratch (scan_scratch(n) ints)
-cudaError_t launch_tile_scan(const int* count, int ntiles, int* start, int* cursor, int* scratch,
-                             cudaStream_t st, int pdl);
+cudaError_t launch_tile_count(const SortParams& P, const SortSet& Q, cudaStream_t st);
+// exclusive scan of every species' count[0..bins) into start[0..bins] and
+// cursor; more than 4096 bins take three launches and the scratch
+cudaError_t launch_tile_scan(const SortSet& Q, int bins, cudaStream_t st, int pdl);
 inline long long scan_scratch(long long n) { return 3 * ((n + 4095) / 4096 + 1); }
-// arrays with rows of ld elements, the first n of which are particles
-// perm (or null): perm[new slot] = old slot
-cudaError_t launch_tile_scatter(const SortParams& P, const int* cell, const float* off,
-                                const float* u, long long n, long long ld, int* cursor,
-                                int* cell_out, float* off_out, float* u_out, cudaStream_t st,
-                                int* perm = nullptr);
+cudaError_t launch_tile_scatter(const SortParams& P, const SortSet& Q, cudaStream_t st);
 // bucket starts t[0..nb] from outside: unless they are a partition of [0, n)
 // they become one bucket, and ST_BAD_BUCKETS is set
 // out[i] = tstart[i] clamped to [lo, hi) for i < nb1 (one slot range's buckets)

@@ -64,9 +64,14 @@ __device__ __forceinline__ int warp_reserve(int* counter, int key, unsigned acti
 // match_any first took 60 us against 43 for 16.8 M particles.
 constexpr int kCountSlots = 1024;
 template <int D>
-__global__ void __launch_bounds__(256) k_tile_count(const SortParams P, const int* __restrict__ cell,
-                                                    long long n, long long chunk, int* count) {
+__global__ void __launch_bounds__(256) k_tile_count(const SortParams P, const SortSet Q,
+                                                    long long chunk) {
   grid_dependency();
+  const int* __restrict__ cell = Q.sp[blockIdx.y].cell;
+  int* const count = Q.sp[blockIdx.y].count;
+  const long long n = Q.sp[blockIdx.y].n;
+  const long long lo = (long long)blockIdx.x * chunk;
+  if (lo >= n) return;  // a smaller species than another of the launch
   __shared__ int skey[kCountSlots];
   __shared__ int scnt[kCountSlots];
   for (int s = threadIdx.x; s < kCountSlots; s += blockDim.x) {
@@ -74,7 +79,6 @@ __global__ void __launch_bounds__(256) k_tile_count(const SortParams P, const in
     scnt[s] = 0;
   }
   __syncthreads();
-  const long long lo = (long long)blockIdx.x * chunk;
   const long long hi = lo + chunk < n ? lo + chunk : n;
   constexpr int U = 4;  // rounds whose loads are issued together (4 loads in flight per thread)
   for (long long base = lo; base < hi; base += U * blockDim.x) {  // block-uniform trip count
@@ -104,10 +108,14 @@ __global__ void __launch_bounds__(256) k_tile_count(const SortParams P, const in
 }
 
 // Exclusive scan of count[0..ntiles) into start[0..ntiles] (start[ntiles] =
-// total) and cursor = start, in one block of 1024 threads.
-__global__ void __launch_bounds__(1024) k_tile_scan(const int* __restrict__ count, int ntiles,
-                                                    int* start, int* cursor) {
+// total) and cursor = start, in one block of 1024 threads per species; with
+// parts, of the multi-block form's block totals instead (ntiles of them).
+__global__ void __launch_bounds__(1024) k_tile_scan(const SortSet Q, int ntiles, int parts) {
   grid_dependency();
+  const SortSpecies& S = Q.sp[blockIdx.x];
+  const int* count = parts ? S.scratch : S.count;
+  int* start = parts ? S.scratch + ntiles : S.start;
+  int* cursor = parts ? S.scratch + 2 * ntiles + 1 : S.cursor;
   __shared__ int warp_sums[32];
   __shared__ int carry;
   if (threadIdx.x == 0) carry = 0;
@@ -151,9 +159,11 @@ __global__ void __launch_bounds__(1024) k_tile_scan(const int* __restrict__ coun
 // total in part[]; one block scans part[]; every block then adds its offset
 // (start[bins] = total, cursor = start).
 constexpr int kScanChunk = 4096;  // counts per block: 4 per thread of 1024
-__global__ void __launch_bounds__(1024) k_scan_chunks(const int* __restrict__ count, int n,
-                                                      int* start, int* part) {
+__global__ void __launch_bounds__(1024) k_scan_chunks(const SortSet Q, int n) {
   grid_dependency();
+  const int* __restrict__ count = Q.sp[blockIdx.y].count;
+  int* start = Q.sp[blockIdx.y].start;
+  int* part = Q.sp[blockIdx.y].scratch;
   __shared__ int warp_sums[32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int base = blockIdx.x * kScanChunk + 4 * threadIdx.x;
@@ -190,9 +200,11 @@ __global__ void __launch_bounds__(1024) k_scan_chunks(const int* __restrict__ co
   if (threadIdx.x == 1023) part[blockIdx.x] = run;
 }
 
-__global__ void __launch_bounds__(1024) k_scan_add(int* start, int* cursor, int n,
-                                                   const int* part_scan) {
+__global__ void __launch_bounds__(1024) k_scan_add(const SortSet Q, int n) {
   grid_dependency();
+  int* start = Q.sp[blockIdx.y].start;
+  int* cursor = Q.sp[blockIdx.y].cursor;
+  const int* part_scan = Q.sp[blockIdx.y].scratch + gridDim.x;
   const int off = part_scan[blockIdx.x];
   const int base = blockIdx.x * kScanChunk + 4 * threadIdx.x;
 #pragma unroll
@@ -206,13 +218,21 @@ __global__ void __launch_bounds__(1024) k_scan_add(int* start, int* cursor, int 
   if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) start[n] = part_scan[gridDim.x];
 }
 
+#define SORT_SPECIES_ARRAYS(S)                \
+  const int* __restrict__ cell = S.cell;      \
+  const float* __restrict__ off = S.off;      \
+  const float* __restrict__ u = S.u;          \
+  const long long n = S.n, ld = S.ld;         \
+  int* cursor = S.cursor;                     \
+  int* __restrict__ cell_out = S.cell_out;    \
+  float* __restrict__ off_out = S.off_out;    \
+  float* __restrict__ u_out = S.u_out;        \
+  int* __restrict__ perm = S.perm;
+
 template <int D>
-__global__ void k_tile_scatter_lanes(const SortParams P, const int* __restrict__ cell,
-                               const float* __restrict__ off, const float* __restrict__ u,
-                               long long n, long long ld, int* cursor, int* __restrict__ cell_out,
-                               float* __restrict__ off_out, float* __restrict__ u_out,
-                               int* __restrict__ perm) {
+__global__ void k_tile_scatter_lanes(const SortParams P, const SortSet Q) {
   grid_dependency();
+  SORT_SPECIES_ARRAYS(Q.sp[blockIdx.y])
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long base = (long long)blockIdx.x * blockDim.x; base < n; base += stride) {
     const long long p = base + threadIdx.x;
@@ -243,12 +263,11 @@ __global__ void k_tile_scatter_lanes(const SortParams P, const int* __restrict__
 // warp's equal bins first took 202 us); a particle whose table slot another
 // bin holds reserves its place in the global cursor by itself.
 template <int D, int U>
-__global__ void __launch_bounds__(256) k_tile_scatter(
-    const SortParams P, const int* __restrict__ cell, const float* __restrict__ off,
-    const float* __restrict__ u, long long n, long long ld, int* cursor, int* __restrict__ cell_out,
-    float* __restrict__ off_out, float* __restrict__ u_out, int* __restrict__ perm) {
+__global__ void __launch_bounds__(256) k_tile_scatter(const SortParams P, const SortSet Q) {
   grid_dependency();
   constexpr int kChunk = 256 * U;
+  SORT_SPECIES_ARRAYS(Q.sp[blockIdx.y])
+  if ((long long)blockIdx.x * kChunk >= n) return;  // a smaller species than another of the launch
   __shared__ int skey[kCountSlots];  // bin of a table slot, then the bin's reserved global slot
   __shared__ int scnt[kCountSlots];  // its particles here, then their first place in bin order
   __shared__ int sdst[kChunk];       // global slot of each place in bin order
@@ -380,61 +399,63 @@ static unsigned blocks_for(long long n) {
   return (unsigned)(b < 1 ? 1 : b);
 }
 
-cudaError_t launch_tile_count(const SortParams& P, const int* cell, long long n, int* count,
-                              cudaStream_t st) {
+// The species of a sort share its launches: on small boxes a launch, not the
+// work, is what a sort costs (1D box of 2 x 32,768 particles, a sort every 10
+// steps, 20 steps: 188 -> 165 us; 2 x 707,560 2D ones 914 -> 886; with smaller
+// chunks for the count).
+static long long most_particles(const SortSet& Q) {
+  long long n = 0;
+  for (int s = 0; s < Q.ns; ++s) n = std::max(n, Q.sp[s].n);
+  return n;
+}
+
+cudaError_t launch_tile_count(const SortParams& P, const SortSet& Q, cudaStream_t st) {
+  const long long n = most_particles(Q);
   if (n == 0) return cudaSuccess;
   const int pdl = P.g.pdl;
-  // contiguous chunks of at least 4096 particles (a multiple of 256), at most
-  // 16 blocks per SM
-  long long nb = (n + 4095) / 4096;
+  // contiguous chunks of 4096 particles or more (a multiple of 256), at most 16
+  // blocks per SM; down to 1024 where that leaves SMs without a block
+  long long nb = std::max((n + 4095) / 4096, std::min((n + 1023) / 1024, 152LL));
   if (nb > 152LL * 16) nb = 152LL * 16;
   const long long chunk = ((n + nb - 1) / nb + 255) / 256 * 256;
-  nb = (n + chunk - 1) / chunk;
+  const dim3 grid((unsigned)((n + chunk - 1) / chunk), Q.ns);
   switch (P.g.dim) {
-    case 1: launch_kernel(pdl, k_tile_count<1>, (unsigned)nb, 256, 0, st, P, cell, n, chunk, count); break;
-    case 2: launch_kernel(pdl, k_tile_count<2>, (unsigned)nb, 256, 0, st, P, cell, n, chunk, count); break;
-    case 3: launch_kernel(pdl, k_tile_count<3>, (unsigned)nb, 256, 0, st, P, cell, n, chunk, count); break;
+    case 1: launch_kernel(pdl, k_tile_count<1>, grid, 256, 0, st, P, Q, chunk); break;
+    case 2: launch_kernel(pdl, k_tile_count<2>, grid, 256, 0, st, P, Q, chunk); break;
+    case 3: launch_kernel(pdl, k_tile_count<3>, grid, 256, 0, st, P, Q, chunk); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
 }
 
-cudaError_t launch_tile_scan(const int* count, int ntiles, int* start, int* cursor, int* scratch,
-                             cudaStream_t st, int pdl) {
-  if (ntiles <= kScanChunk) {
-    launch_kernel(pdl, k_tile_scan, 1, 1024, 0, st, count, ntiles, start, cursor);
+cudaError_t launch_tile_scan(const SortSet& Q, int bins, cudaStream_t st, int pdl) {
+  if (bins <= kScanChunk) {
+    launch_kernel(pdl, k_tile_scan, Q.ns, 1024, 0, st, Q, bins, 0);
     return cudaGetLastError();
   }
   // scratch: block totals [nb], their scan [nb + 1], the scan's cursor [nb]
-  const int nb = (ntiles + kScanChunk - 1) / kScanChunk;
-  int* part = scratch;
-  int* part_scan = scratch + nb;
-  int* part_cursor = scratch + 2 * nb + 1;
-  launch_kernel(pdl, k_scan_chunks, nb, 1024, 0, st, count, ntiles, start, part);
-  launch_kernel(pdl, k_tile_scan, 1, 1024, 0, st, part, nb, part_scan, part_cursor);
-  launch_kernel(pdl, k_scan_add, nb, 1024, 0, st, start, cursor, ntiles, part_scan);
+  const int nb = (bins + kScanChunk - 1) / kScanChunk;
+  launch_kernel(pdl, k_scan_chunks, dim3(nb, Q.ns), 1024, 0, st, Q, bins);
+  launch_kernel(pdl, k_tile_scan, Q.ns, 1024, 0, st, Q, nb, 1);
+  launch_kernel(pdl, k_scan_add, dim3(nb, Q.ns), 1024, 0, st, Q, bins);
   return cudaGetLastError();
 }
 
-cudaError_t launch_tile_scatter(const SortParams& P, const int* cell, const float* off,
-                                const float* u, long long n, long long ld, int* cursor,
-                                int* cell_out, float* off_out, float* u_out, cudaStream_t st,
-                                int* perm) {
+cudaError_t launch_tile_scatter(const SortParams& P, const SortSet& Q, cudaStream_t st) {
+  const long long n = most_particles(Q);
   if (n == 0) return cudaSuccess;
   const int pdl = P.g.pdl;
   const auto launch = [&](auto kernel, int chunk) {
-    return launch_kernel(pdl, kernel, (unsigned)((n + chunk - 1) / chunk), 256, 0, st, P, cell, off, u,
-                         n, ld, cursor, cell_out, off_out, u_out, perm);
+    return launch_kernel(pdl, kernel, dim3((unsigned)((n + chunk - 1) / chunk), Q.ns), 256, 0, st,
+                         P, Q);
   };
   // few particles: the lanes kernel, whose blocks of 256 spread them over more
   // of the chip (65,536 2D particles, whole sort: 70 us against 78 with 1024 to
   // a block; 262,144: 83 against 79, and 83 with 2048; 1.05 M: 133, 115, 111)
   const bool few = n < 1 << 17, some = n < 1 << 19;
-  const unsigned nb = blocks_for(n);
-#define PIC_SCATTER(D)                                                                        \
-  if (few)                                                                                    \
-    return launch_kernel(pdl, k_tile_scatter_lanes<D>, nb, 256, 0, st, P, cell, off, u, n, ld, \
-                         cursor, cell_out, off_out, u_out, perm);                             \
+  const dim3 grid(blocks_for(n), Q.ns);
+#define PIC_SCATTER(D)                                                                     \
+  if (few) return launch_kernel(pdl, k_tile_scatter_lanes<D>, grid, 256, 0, st, P, Q);     \
   return some ? launch(k_tile_scatter<D, 4>, 1024) : launch(k_tile_scatter<D, 8>, 2048);
   switch (P.g.dim) {
     case 1: PIC_SCATTER(1)

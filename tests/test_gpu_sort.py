@@ -90,3 +90,43 @@ def test_adopted_bucket_starts_are_checked(tile):
         sim.check()
     assert e.value.status == B.PIC_ERR_STATE
     sim.close()
+
+
+@pytest.mark.parametrize("counts", [(70_000, 0, 5), (3, 140_000, 1025), (600_000, 2049, 131_072, 0)])
+@pytest.mark.parametrize("dim,shape,tile", [(1, (4000, 1, 1), None), (2, (203, 97, 1), None),
+                                            (2, (256, 256, 1), [2, 2]), (3, (41, 33, 30), None)])
+def test_species_of_different_size_in_one_sort(dim, shape, tile, counts):
+    """Every species of a sort, whose launches they share (the largest one's
+    size sets them): records bit for bit and the starts the bins' counts."""
+    import torch
+
+    from paper_1906_06306_gb300 import Simulation
+    from paper_1906_06306_gb300 import binding as B
+
+    rs = np.random.default_rng(sum(counts) + dim)
+    cells = shape[0] * shape[1] * shape[2]
+    sp = [dict(q=1.0, m=1.0, cell=rs.integers(0, cells, n).astype(np.int32),
+               off=rs.random((dim, n), dtype=np.float32), u=rs.normal(size=(3, n)).astype(np.float32)) for n in counts]
+    sim = Simulation(dim, *shape, 0.45, np.zeros((9,) + shape[::-1], np.float32), sp,
+                     tuning=dict(tile=tile) if tile else None)
+    for d, s in zip(sim.species, sp):
+        for k in ("cell", "off", "u"):
+            d[k][..., : d["n"]] = torch.from_numpy(s[k]).to(sim.device)
+    nb = B.pic_sort_bins(sim.ctx)
+    perm = [torch.full((max(n, 1),), -1, dtype=torch.int32, device=sim.device) for n in counts]
+    start = [torch.full((nb + 1,), -1, dtype=torch.int32, device=sim.device) for _ in counts]
+    B.pic_sort_record(sim.ctx, [p.data_ptr() for p in perm], [t.data_ptr() for t in start])
+    sim.check()
+    for got, s, p, t, n in zip(sim.download()[1], sp, perm, start, counts):
+        if n == 0:
+            continue
+        p, t = p.cpu().numpy(), t.cpu().numpy()
+        assert np.array_equal(np.sort(p), np.arange(n))
+        for k in ("cell", "off", "u"):
+            assert np.array_equal(got[k].view(np.int32), s[k][..., p].view(np.int32))
+        assert t[0] == 0 and t[-1] == n and (np.diff(t) >= 0).all()
+        bin_of = np.repeat(np.arange(nb), np.diff(t))
+        order = np.argsort(got["cell"], kind="stable")
+        c, b = got["cell"][order], bin_of[order]
+        assert (b[1:] == b[:-1])[c[1:] == c[:-1]].all()
+    sim.close()
