@@ -1031,6 +1031,7 @@ def run_batched(args):
     launches = 0
     for sm in sims:
         per_step, per_sort = launches_per_step(sm)
+        per_step, per_sort = per_step - fused_away(sm), per_sort - sort_shared(sm)
         per_step -= fused_away(sm)
         launches += args.steps * per_step + -(-args.steps // sm.tuning()["sort_every"]) * per_sort
     line = {
