@@ -1031,8 +1031,8 @@ def run_batched(args):
     launches = 0
     for sm in sims:
         per_step, per_sort = launches_per_step(sm)
-        per_step, per_sort = per_step - fused_away(sm), per_sort - sort_shared(sm)
         per_step -= fused_away(sm)
+        per_sort -= sort_shared(sm)
         launches += args.steps * per_step + -(-args.steps // sm.tuning()["sort_every"]) * per_sort
     line = {
         "metric": METRIC, "value": value, "unit": "particle-steps/s", "n_gpus": world,
