@@ -236,8 +236,9 @@ __global__ void k_rho(const GridDev g, const int* __restrict__ cell, const float
 // FP64 atomics of k_rho, and so does the unsorted tail.  The global atomics
 // bounded that kernel (one FP64 atomic per L2 slice and clock: 4 a particle,
 // 338 us for 16.8 M in 2D); here a block issues one per window node, and the
-// kernel takes 95 us, bound by the 10 shared atomics a particle.  Four rounds
-// of loads go out together (135 us with one).
+// kernel takes 87 us, bound by instruction issue and 8 shared atomics a
+// particle (96 us with all moments by 64-bit shifts and 10 atomics).  Four
+// rounds of loads go out together (135 us with one).
 constexpr int kRhoBatch = 1 << 15;
 
 template <int D>
@@ -273,15 +274,16 @@ __global__ void __launch_bounds__(256, 6) k_rho_tiles(const GridDev g, const Til
     for (int w = threadIdx.x; w < NW * wc; w += blockDim.x) sw[w] = 0u;
     __syncthreads();
     constexpr int U = 4;  // rounds whose loads are issued together
-    for (long long base = first + threadIdx.x; base < last; base += U * blockDim.x) {
+    const int here = (int)(last - first);
+    for (int base = threadIdx.x; base < here; base += U * blockDim.x) {
       int cu[U];
       float ou[U][2];
 #pragma unroll
       for (int r = 0; r < U; ++r) {
-        const long long p = base + r * blockDim.x;
-        cu[r] = p < last ? cell[p] : -1;
-        ou[r][0] = p < last ? off[p] : 0.f;
-        ou[r][1] = D == 2 && p < last ? off[ld + p] : 0.f;
+        const int p = base + r * blockDim.x;
+        cu[r] = p < here ? cell[first + p] : -1;
+        ou[r][0] = p < here ? off[first + p] : 0.f;
+        ou[r][1] = D == 2 && p < here ? off[ld + first + p] : 0.f;
       }
 #pragma unroll
       for (int r = 0; r < U; ++r) {
@@ -301,22 +303,49 @@ __global__ void __launch_bounds__(256, 6) k_rho_tiles(const GridDev g, const Til
         if (D == 2) in &= l1 < W1 - 1 && o[1] >= 0.f && o[1] < 1.f;
         if (in) {
           unsigned* s = sw + l0 + W0 * l1;
-          unsigned long long m[3];
-          const unsigned mx = mantissa(o[0]);
-          const int ex = exponent(o[0]) - 102;  // units of 2^-48
-          m[0] = shifted(mx, ex);
-          if (D == 2) {
-            const unsigned my = mantissa(o[1]);
-            const int ey = exponent(o[1]) - 150;
-            m[1] = shifted(my, ey + 48);
-            m[2] = shifted((unsigned long long)mx * my, ex + ey);
+          // the moments' 16-bit limbs in units of 2^-48, last first: offsets of
+          // 2^-8 or more are whole in units of 2^-32
+          unsigned m[3][3];
+          if (o[0] >= 0x1p-8f && (D == 1 || o[1] >= 0x1p-8f)) {
+            const unsigned x = __float2uint_rz(o[0] * 0x1p32f);
+            m[0][0] = 0u;
+            m[0][1] = x & 0xffffu;
+            m[0][2] = x >> 16;
+            if (D == 2) {
+              const unsigned y = __float2uint_rz(o[1] * 0x1p32f);
+              const unsigned long long xy = (unsigned long long)x * y;  // units of 2^-64
+              m[1][0] = 0u;
+              m[1][1] = y & 0xffffu;
+              m[1][2] = y >> 16;
+              m[2][0] = (unsigned)xy >> 16;
+              m[2][1] = (unsigned)(xy >> 32) & 0xffffu;
+              m[2][2] = (unsigned)(xy >> 48);
+            }
+          } else {
+            unsigned long long v[3];
+            const unsigned mx = mantissa(o[0]);
+            const int ex = exponent(o[0]) - 102;
+            v[0] = shifted(mx, ex);
+            if (D == 2) {
+              const unsigned my = mantissa(o[1]);
+              const int ey = exponent(o[1]) - 150;
+              v[1] = shifted(my, ey + 48);
+              v[2] = shifted((unsigned long long)mx * my, ex + ey);
+            }
+#pragma unroll
+            for (int k = 0; k < (1 << D) - 1; ++k) {
+              m[k][0] = (unsigned)v[k] & 0xffffu;
+              m[k][1] = (unsigned)v[k] >> 16;
+              m[k][2] = (unsigned)(v[k] >> 32);
+            }
           }
           atomicAdd(s, 1u);
-  #pragma unroll
+#pragma unroll
           for (int k = 0; k < (1 << D) - 1; ++k) {
-            atomicAdd(s + (1 + 3 * k) * wc, (unsigned)m[k] & 0xffffu);
-            atomicAdd(s + (2 + 3 * k) * wc, (unsigned)m[k] >> 16);
-            atomicAdd(s + (3 + 3 * k) * wc, (unsigned)(m[k] >> 32));
+            // few warps have a last limb of w_x or w_y to add
+            if (k == 2 || m[k][0] != 0u) atomicAdd(s + (1 + 3 * k) * wc, m[k][0]);
+            atomicAdd(s + (2 + 3 * k) * wc, m[k][1]);
+            atomicAdd(s + (3 + 3 * k) * wc, m[k][2]);
           }
         } else {
           rho_particle<D>(g, c, o, q, rho);
