@@ -1,9 +1,9 @@
-// FDTD2 field update and Binomial2 current filter (arXiv:1906.06306,
-// Sect. 2.3.1, Eqs. (fdE), (fdB), Table 2) on periodic Yee planes.
-// One thread per lattice point, x fastest, so every plane is streamed with
-// coalesced loads; neighbours one point away come from the same or adjacent
-// rows and hit L1/L2.  The filter runs as one 3-point sub-pass per gridded
-// axis (x, then y, then z), the order in which the paper's filter is applied.
+// FDTD2 and FDTD4 field updates (arXiv:1906.06306, Sect. 2.3.1, Eqs. (fdE),
+// (fdB), Table 2) on periodic Yee planes, and the FP64 form of the Binomial2
+// filter's sub-pass (the current's filter: pic_filter.cu).
+// One thread per lattice point (or four), x fastest, so every plane is streamed
+// with coalesced loads; neighbours one point away come from the same or adjacent
+// rows and hit L1/L2.
 #include "pic_kernels.h"
 
 namespace pic {

@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(128) k_filter_y2(const float* __restrict__ src
 // the last three y results for the z sub-pass.  Reads: the column, its (x, y)
 // halo (rows of neighbouring columns, mostly from L2) and two extra planes per
 // run; writes: the column, 16 bytes per store.  Every output goes through the
-// same arithmetic, in the same order, as three k_filter_axis sub-passes.
+// x, y and z sub-passes in this order, with the arithmetic of the marched forms.
 // Grid: x = column index + columns x run, y = plane.
 constexpr int ZX = 128, ZY = 16, ZS = 4;
 constexpr int ZROW = ZX + 8;  // stage row: [3] left halo, [4, 4 + ZX) interior, [4 + ZX] right
