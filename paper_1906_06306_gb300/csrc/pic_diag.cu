@@ -228,10 +228,12 @@ __global__ void k_rho(const GridDev g, const int* __restrict__ cell, const float
 // every particle are differences of these (w_x - w_x w_y, ...), so a node's
 // charge is one integer sum over its four cells, rounded once to FP64.
 // Each moment goes as three 16-bit limbs into 32-bit words with native
-// integer atomics (64-bit shared atomics are a compare-and-swap loop), so
-// kRhoBatch = 2^15 particles can neither overflow a word nor the 64-bit
-// sums.  An offset has 24 significant bits: a moment is short of its exact
-// value by less than 2^-47, below the rounding of an FP64 sum of 16 charges.
+// integer atomics (64-bit shared atomics are a compare-and-swap loop).  A word
+// holds 2^16 such limbs, but the count in units of 2^-48 is a signed 64-bit
+// sum, which 2^15 particles of one node overflow: the window is folded and
+// cleared after every kRhoBatch = 2^14 particles.  An offset has 24 significant
+// bits: a moment is short of its exact value by less than 2^-47, below the
+// rounding of an FP64 sum of 16 charges.
 // Particles outside the window, or whose offsets are not in [0, 1), take the
 // FP64 atomics of k_rho, and so does the unsorted tail.  The global atomics
 // bounded that kernel (one FP64 atomic per L2 slice and clock: 4 a particle,
@@ -239,7 +241,7 @@ __global__ void k_rho(const GridDev g, const int* __restrict__ cell, const float
 // kernel takes 87 us, bound by instruction issue and 8 shared atomics a
 // particle (96 us with all moments by 64-bit shifts and 10 atomics).  Four
 // rounds of loads go out together (135 us with one).
-constexpr int kRhoBatch = 1 << 15;
+constexpr int kRhoBatch = 1 << 14;
 
 template <int D>
 __host__ __device__ constexpr int rho_words() {

@@ -1,0 +1,56 @@
+"""The charge behind pic_energies' Gauss residual where many particles share one
+cell: the tile kernel's batches, and the sums that their words must hold."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+Q = np.float32(0.01)
+
+
+def _box(dim, cell, off, tile=8):
+    """One species at rest in a box of 64 tiles without fields: the residual is the charge."""
+    from paper_1906_06306_gb300 import Simulation
+
+    n = (512, 1, 1) if dim == 1 else (64, 64, 1)
+    sp = dict(q=Q, m=1.0, cell=cell, off=off, u=np.zeros((3, cell.size), dtype=np.float32))
+    sim = Simulation(dim, *n, 0.45, np.zeros((9,) + n[::-1], dtype=np.float32), [sp],
+                     tuning=dict(tile=[tile] * dim + [1] * (3 - dim)))
+    sim.sort()
+    return sim
+
+
+def _node_charges(off):
+    """Charge of the corner nodes of the one cell that holds every particle, extended precision."""
+    L = np.longdouble
+    w = off.astype(L)
+    out = []
+    for corner in range(1 << w.shape[0]):
+        t = L(1.0)
+        for d in range(w.shape[0]):
+            t = t * (w[d] if corner >> d & 1 else 1 - w[d])
+        out.append(L(Q) * (t * np.ones(off.shape[1], dtype=L)).sum())
+    return np.array(out)
+
+
+@pytest.mark.parametrize("offset", [0.0, 2.0 ** -50, 0.25, 1.0 - 2.0 ** -24])
+@pytest.mark.parametrize("n", [32_768, 70_000])
+@pytest.mark.parametrize("dim", [1, 2])
+def test_full_batches_in_one_cell(dim, n, offset):
+    # a share of 32,768 particles or more, far above the mean of the tiles, from one block
+    off = np.full((dim, n), offset, dtype=np.float32)
+    cell = np.full(n, 300 if dim == 1 else 30 + 64 * 21, dtype=np.int32)
+    sim = _box(dim, cell, off)
+    ref = _node_charges(off)
+    # E at the cell's low corner carries the sign: div E = +q n there, residual = q n - rho
+    sim.fields[0].view(-1)[int(cell[0])] = float(ref[0])
+    lo = float(np.float32(float(ref[0])))
+    nodes = {0: lo - float(ref[0])}
+    for k in range(1, 1 << dim):
+        nodes[k] = -float(ref[k])
+    nodes[1] -= lo  # the x neighbour's divergence takes E off again
+    got = sim.energies()
+    want = max(abs(v) for v in nodes.values())
+    # each particle's weights within 2^-46 of their exact values, FP64 sums
+    assert abs(got[3] - want) <= 2.0 ** -46 * float(Q) * n
+    sim.close()
