@@ -224,38 +224,30 @@ __global__ void k_rho(const GridDev g, const int* __restrict__ cell, const float
 // The same charge for particles grouped by tile (1D and 2D), by fixed-point
 // sums in shared memory.  A block takes its share of a tile's bucket and sums,
 // for each cell of the tile's window, the particle count and the moments
-// sum w_x, sum w_y, sum w_x w_y in units of 2^-48; the four corner weights of
-// every particle are differences of these (w_x - w_x w_y, ...), so a node's
-// charge is one integer sum over its four cells, rounded once to FP64.
-// Each moment goes as three 16-bit limbs into 32-bit words with native
-// integer atomics (64-bit shared atomics are a compare-and-swap loop).  A word
-// holds 2^16 such limbs, but the count in units of 2^-48 is a signed 64-bit
-// sum, which 2^15 particles of one node overflow: the window is folded and
-// cleared after every kRhoBatch = 2^14 particles.  An offset has 24 significant
-// bits: a moment is short of its exact value by less than 2^-47, below the
-// rounding of an FP64 sum of 16 charges.
-// Particles outside the window, or whose offsets are not in [0, 1), take the
-// FP64 atomics of k_rho, and so does the unsorted tail.  The global atomics
-// bounded that kernel (one FP64 atomic per L2 slice and clock: 4 a particle,
-// 338 us for 16.8 M in 2D); here a block issues one per window node, and the
-// kernel takes 87 us, bound by instruction issue and 8 shared atomics a
-// particle (96 us with all moments by 64-bit shifts and 10 atomics).  Four
-// rounds of loads go out together (135 us with one).
+// sum w_x, sum w_y, sum w_x w_y; the four corner weights of every particle are
+// differences of these (w_x - w_x w_y, ...), so a node's charge is one integer
+// sum over its four cells, rounded once to FP64.
+// Nothing is cut off: an offset of 2^-8 or more (or 0) is whole in units of
+// 2^-31, a product of two in units of 2^-62, and the node sums take 128-bit
+// integers.  Each moment goes as 16-bit limbs into 32-bit words with native
+// integer atomics (64-bit shared atomics are a compare-and-swap loop);
+// kRhoBatch = 2^14 particles, a quarter of what a word holds, go between two
+// folds.  Particles outside the window, or with other offsets (0.8 % of
+// uniform ones on two axes), are queued and take the FP64 atomics of k_rho
+// together, and so does the unsorted tail.  The global atomics bounded that
+// kernel (one FP64 atomic per L2 slice and clock: 4 a particle, 338 us for
+// 16.8 M in 2D); here a block issues one per window node, and the kernel takes
+// 93 us, bound by instruction issue and 9 shared atomics a particle (87 us with
+// moments cut at 2^-48, 8 atomics).  Four rounds of loads go out together.
 constexpr int kRhoBatch = 1 << 14;
+constexpr int kRhoQueue = 1024;
 
 template <int D>
 __host__ __device__ constexpr int rho_words() {
-  return 1 + 3 * ((1 << D) - 1);
+  return D == 1 ? 3 : 9;  // count; w_x, w_y in two limbs each; w_x w_y in four
 }
 
-// A float w in [0, 1) is m 2^(e - 150), m < 2^24.
-__device__ __forceinline__ unsigned mantissa(float w) {
-  return (__float_as_uint(w) & 0x7fffffu) | 0x800000u;
-}
-__device__ __forceinline__ int exponent(float w) { return (int)((__float_as_uint(w) >> 23) & 255u); }
-__device__ __forceinline__ unsigned long long shifted(unsigned long long m, int sh) {
-  return sh >= 0 ? m << sh : (sh > -64 ? m >> -sh : 0ULL);
-}
+__device__ __forceinline__ bool rho_whole(float w) { return (w >= 0x1p-8f && w < 1.0f) || w == 0.f; }
 
 template <int D>
 __global__ void __launch_bounds__(256, 6) k_rho_tiles(const GridDev g, const TileDev t, int splits,
@@ -264,6 +256,8 @@ __global__ void __launch_bounds__(256, 6) k_rho_tiles(const GridDev g, const Til
                                                    const float* __restrict__ off, long long ld,
                                                    double q, double* rho) {
   extern __shared__ unsigned sw[];
+  __shared__ unsigned short queue[kRhoQueue];  // particles of the batch for the FP64 atomics
+  __shared__ int queued;
   constexpr int NW = rho_words<D>();
   const int tile = blockIdx.x / splits, split = blockIdx.x - tile * splits;
   const int w0[2] = {(tile % t.nt[0]) * t.T[0] - t.H, D == 2 ? (tile / t.nt[0]) * t.T[1] - t.H : 0};
@@ -274,6 +268,7 @@ __global__ void __launch_bounds__(256, 6) k_rho_tiles(const GridDev g, const Til
   for (long long first = a; first < b; first += kRhoBatch) {
     const long long last = first + kRhoBatch < b ? first + kRhoBatch : b;
     for (int w = threadIdx.x; w < NW * wc; w += blockDim.x) sw[w] = 0u;
+    if (threadIdx.x == 0) queued = 0;
     __syncthreads();
     constexpr int U = 4;  // rounds whose loads are issued together
     const int here = (int)(last - first);
@@ -301,89 +296,76 @@ __global__ void __launch_bounds__(256, 6) k_rho_tiles(const GridDev g, const Til
           l0 = wrapi(l0, g.n[0]);
           if (D == 2) l1 = wrapi(l1, g.n[1]);
         }
-        bool in = l0 < W0 - 1 && o[0] >= 0.f && o[0] < 1.f;
-        if (D == 2) in &= l1 < W1 - 1 && o[1] >= 0.f && o[1] < 1.f;
+        bool in = l0 < W0 - 1 && rho_whole(o[0]);
+        if (D == 2) in &= l1 < W1 - 1 && rho_whole(o[1]);
         if (in) {
           unsigned* s = sw + l0 + W0 * l1;
-          // the moments' 16-bit limbs in units of 2^-48, last first: offsets of
-          // 2^-8 or more are whole in units of 2^-32
-          unsigned m[3][3];
-          if (o[0] >= 0x1p-8f && (D == 1 || o[1] >= 0x1p-8f)) {
-            const unsigned x = __float2uint_rz(o[0] * 0x1p32f);
-            m[0][0] = 0u;
-            m[0][1] = x & 0xffffu;
-            m[0][2] = x >> 16;
-            if (D == 2) {
-              const unsigned y = __float2uint_rz(o[1] * 0x1p32f);
-              const unsigned long long xy = (unsigned long long)x * y;  // units of 2^-64
-              m[1][0] = 0u;
-              m[1][1] = y & 0xffffu;
-              m[1][2] = y >> 16;
-              m[2][0] = (unsigned)xy >> 16;
-              m[2][1] = (unsigned)(xy >> 32) & 0xffffu;
-              m[2][2] = (unsigned)(xy >> 48);
-            }
-          } else {
-            unsigned long long v[3];
-            const unsigned mx = mantissa(o[0]);
-            const int ex = exponent(o[0]) - 102;
-            v[0] = shifted(mx, ex);
-            if (D == 2) {
-              const unsigned my = mantissa(o[1]);
-              const int ey = exponent(o[1]) - 150;
-              v[1] = shifted(my, ey + 48);
-              v[2] = shifted((unsigned long long)mx * my, ex + ey);
-            }
-#pragma unroll
-            for (int k = 0; k < (1 << D) - 1; ++k) {
-              m[k][0] = (unsigned)v[k] & 0xffffu;
-              m[k][1] = (unsigned)v[k] >> 16;
-              m[k][2] = (unsigned)(v[k] >> 32);
-            }
-          }
+          const unsigned x = __float2uint_rz(o[0] * 0x1p31f);
           atomicAdd(s, 1u);
-#pragma unroll
-          for (int k = 0; k < (1 << D) - 1; ++k) {
-            // few warps have a last limb of w_x or w_y to add
-            if (k == 2 || m[k][0] != 0u) atomicAdd(s + (1 + 3 * k) * wc, m[k][0]);
-            atomicAdd(s + (2 + 3 * k) * wc, m[k][1]);
-            atomicAdd(s + (3 + 3 * k) * wc, m[k][2]);
+          atomicAdd(s + wc, x & 0xffffu);
+          atomicAdd(s + 2 * wc, x >> 16);
+          if (D == 2) {
+            const unsigned y = __float2uint_rz(o[1] * 0x1p31f);
+            const unsigned long long xy = (unsigned long long)x * y;
+            atomicAdd(s + 3 * wc, y & 0xffffu);
+            atomicAdd(s + 4 * wc, y >> 16);
+            atomicAdd(s + 5 * wc, (unsigned)xy & 0xffffu);
+            atomicAdd(s + 6 * wc, (unsigned)xy >> 16);
+            atomicAdd(s + 7 * wc, (unsigned)(xy >> 32) & 0xffffu);
+            atomicAdd(s + 8 * wc, (unsigned)(xy >> 48));
           }
         } else {
-          rho_particle<D>(g, c, o, q, rho);
+          const int slot = atomicAdd(&queued, 1);
+          if (slot < kRhoQueue)
+            queue[slot] = (unsigned short)(base + r * blockDim.x);
+          else
+            rho_particle<D>(g, c, o, q, rho);
         }
       }
     }
     __syncthreads();
+    for (int k = threadIdx.x; k < min(queued, kRhoQueue); k += blockDim.x) {
+      const long long p = first + queue[k];
+      const float o[3] = {off[p], D == 2 ? off[ld + p] : 0.f, 0.f};
+      rho_particle<D>(g, cell[p], o, q, rho);
+    }
     for (int w = threadIdx.x; w < wc; w += blockDim.x) {
       const int lx = w % W0, ly = w / W0;
-      // moments of cell v: {count 2^48, w_x, w_y, w_x w_y}
-      auto cell_sums = [&](int v, long long* m) {
-        m[0] = (long long)sw[v] << 48;
-#pragma unroll
-        for (int k = 0; k < (1 << D) - 1; ++k)
-          m[1 + k] = (long long)sw[v + (1 + 3 * k) * wc] +
-                     ((long long)sw[v + (2 + 3 * k) * wc] << 16) +
-                     ((long long)sw[v + (3 + 3 * k) * wc] << 32);
+      // sums of cell v: {count, w_x, w_y} in units of 2^-31, w_x w_y in 2^-62
+      const auto linear = [&](int v, long long* m) {
+        m[0] = (long long)sw[v] << 31;
+        m[1] = (long long)sw[v + wc] + ((long long)sw[v + 2 * wc] << 16);
+        m[2] = D == 2 ? (long long)sw[v + 3 * wc] + ((long long)sw[v + 4 * wc] << 16) : 0;
       };
-      long long sum = 0, m[4];
-      cell_sums(w, m);
-      sum += D == 1 ? m[0] - m[1] : m[0] - m[1] - m[2] + m[3];
+      const auto product = [&](int v) {
+        const unsigned long long lo = sw[v + 5 * wc] + ((unsigned long long)sw[v + 6 * wc] << 16);
+        const unsigned long long hi = sw[v + 7 * wc] + ((unsigned long long)sw[v + 8 * wc] << 16);
+        return (__int128)lo + ((__int128)hi << 32);
+      };
+      long long sum = 0, m[3];  // units of 2^-31
+      __int128 sum2 = 0;        // units of 2^-62
+      linear(w, m);
+      sum += m[0] - m[1] - m[2];
+      if (D == 2) sum2 += product(w);
       if (lx > 0) {
-        cell_sums(w - 1, m);
-        sum += D == 1 ? m[1] : m[1] - m[3];
+        linear(w - 1, m);
+        sum += m[1];
+        if (D == 2) sum2 -= product(w - 1);
       }
       if (D == 2 && ly > 0) {
-        cell_sums(w - W0, m);
-        sum += m[2] - m[3];
-        if (lx > 0) {
-          cell_sums(w - W0 - 1, m);
-          sum += m[3];
-        }
+        linear(w - W0, m);
+        sum += m[2];
+        sum2 -= product(w - W0);
+        if (lx > 0) sum2 += product(w - W0 - 1);
       }
-      if (sum != 0) {
+      if (D == 2) sum2 += (__int128)sum << 31;
+      if (D == 1 ? sum != 0 : sum2 != 0) {
+        // at most 2^45 and 2^76: all but the last addition are exact
+        const double charge = D == 1 ? (double)sum * 0x1p-31
+                                     : (double)(long long)(sum2 >> 32) * 0x1p-30 +
+                                           (double)(unsigned)sum2 * 0x1p-62;
         const int i = wrapi(w0[0] + lx, g.n[0]), j = D == 2 ? wrapi(w0[1] + ly, g.n[1]) : 0;
-        atomicAdd(&rho[i + (long long)g.n[0] * j], q * ((double)sum * 0x1p-48));
+        atomicAdd(&rho[i + (long long)g.n[0] * j], q * charge);
       }
     }
     __syncthreads();

@@ -54,3 +54,50 @@ def test_full_batches_in_one_cell(dim, n, offset):
     # each particle's weights within 2^-46 of their exact values, FP64 sums
     assert abs(got[3] - want) <= 2.0 ** -46 * float(Q) * n
     sim.close()
+
+
+def _tiny(off):
+    """Particles whose offsets the fixed-point sums do not hold whole: FP64 weights of four roundings."""
+    return int(((off > 0) & (off < 2.0 ** -8)).any(0).sum())
+
+
+def _check_whole(sim, off, cell):
+    ref = _node_charges(off)
+    got = sim.energies()
+    # no fields: one rounding of a batch's sum, one of its product with q and one of its
+    # addition to the node (4 batches at most here); four roundings of each queued
+    # particle's weight and one of its addition
+    batches = 4
+    tol = 2.0 ** -53 * (3 * batches + 5 * _tiny(off)) * float(ref.max())
+    assert abs(got[3] - float(ref.max())) <= tol
+
+
+OFFSETS = [0.0, 2.0 ** -149, 2.0 ** -60, 2.0 ** -30, 2.0 ** -8 - 2.0 ** -32, 2.0 ** -8, 2.0 ** -8 + 2.0 ** -31,
+           0.5, 1.0 - 2.0 ** -24]
+
+
+@pytest.mark.parametrize("dim", [1, 2])
+def test_one_particle_has_all_its_bits(dim):
+    rs = np.random.default_rng(40 + dim)
+    k = np.arange(len(OFFSETS) ** dim)
+    edge = np.array([[OFFSETS[i // len(OFFSETS) ** d % len(OFFSETS)] for i in k] for d in range(dim)])
+    draws = np.minimum(rs.random((dim, 60)).astype(np.float32) * 2.0 ** -rs.integers(0, 12, (dim, 60)),
+                       1 - 2.0 ** -24)
+    cell = np.array([300 if dim == 1 else 30 + 64 * 21], dtype=np.int32)
+    sim = _box(dim, cell, np.zeros((dim, 1), dtype=np.float32))
+    for o in np.concatenate([edge, draws], axis=1).astype(np.float32).T:
+        sim.species[0]["off"][:, :1] = sim.torch.from_numpy(o.reshape(dim, 1)).to(sim.device)
+        _check_whole(sim, o.reshape(dim, 1), cell)
+    sim.close()
+
+
+@pytest.mark.parametrize("n", [1, 255, 1025, 16_384, 40_000])
+@pytest.mark.parametrize("dim", [1, 2])
+def test_many_particles_of_a_cell_have_all_their_bits(dim, n):
+    rs = np.random.default_rng(dim * n)
+    off = np.minimum(rs.random((dim, n)).astype(np.float32), np.float32(1 - 2.0 ** -24))
+    off[:, n // 2:] *= np.float32(2.0 ** -7)  # most of the second half goes through the queue
+    cell = np.full(n, 300 if dim == 1 else 30 + 64 * 21, dtype=np.int32)
+    sim = _box(dim, cell, off)
+    _check_whole(sim, off, cell)
+    sim.close()
