@@ -80,42 +80,105 @@ __device__ __forceinline__ bool df_range(float m) { return m >= kDfMin && m <= k
 
 constexpr int kDfTerms = 16;  // terms summed in double-float before the FP64 sum takes them
 
-// Sums of E^2 and B^2.  Squares are exact in double-float; every 16 points the
-// sums go on in FP64 (1024^2 box: 40 us with FP64 products, 22 us).
+// The GPU's FP64 pipe issues one operation for some thirty FP32 ones, so the
+// diagnostics form their terms and the sums of a thread's terms as sums of three
+// floats, s0 + s1 + s2, each about 2^-24 of the one before: 64 bits and more,
+// where FP64 holds 53.  The error-free sum is Knuth's, the error-free product
+// the fused multiply-add's.  Two values go through each step as the halves of
+// the packed FP32 instructions.
+__device__ __forceinline__ float2 neg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+// a + b = s + the return value
+__device__ __forceinline__ float2 two_sum(float2 a, float2 b, float2& s) {
+  s = add(a, b);
+  const float2 t = add(s, neg(a));
+  return add(add(a, neg(add(s, neg(t)))), add(b, neg(t)));
+}
+// a a = p + the return value
+__device__ __forceinline__ float2 square(float2 a, float2& p) {
+  p = mul(a, a);
+  return fma(a, a, neg(p));
+}
+struct Sum3 {
+  float2 s0, s1, s2;
+  __device__ __forceinline__ void add_term(float2 h, float2 l) {
+    const float2 e = two_sum(s0, h, s0);
+    const float2 f = two_sum(s1, l, s1);
+    const float2 g = two_sum(s1, e, s1);
+    s2 = add(s2, add(f, g));
+  }
+  __device__ __forceinline__ double x() const { return (double)s0.x + ((double)s1.x + s2.x); }
+  __device__ __forceinline__ double y() const { return (double)s0.y + ((double)s1.y + s2.y); }
+};
+// Whether the squares of three floats can be summed this way: the sum of their
+// magnitudes is 0 or between 2^-40 and 2^60 (not for NaN and infinities).
+// Others take FP64.
+__device__ __forceinline__ bool sum3_range(float a, float b, float c) {
+  const float m = fabsf(a) + fabsf(b) + fabsf(c);
+  return (m >= 0x1p-40f && m <= 0x1p60f) || m == 0.f;
+}
+
+constexpr int kSumTerms = 16;  // points or pairs of a thread before its FP64 sum takes them
+
+// not inlined: a branch, not FP64 operations that every thread goes through
+__device__ __noinline__ double squares_fp64(float a, float b, float c) {
+  return (double)a * a + (double)b * b + (double)c * c;
+}
+
+// Sums of E^2 and B^2, one in each half, four points of a thread at a time:
+// 1024^2 box 15 us (FP64 products and sums 40; 38 with the rare FP64 form
+// inlined, which the compiler then evaluates for every point).
 __global__ void k_field_energy(const float* __restrict__ F, long long P, double* acc) {
   __shared__ double sh[32];
   double se = 0.0, sb = 0.0;
-  DF e = {0.f, 0.f}, b = {0.f, 0.f};
-  const long long stride = (long long)gridDim.x * blockDim.x;
+  Sum3 sum = {};
   int terms = 0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P; i += stride) {
-    float v[6];
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  constexpr int U = 4;  // rounds whose loads are issued together
+  for (long long base = blockIdx.x * (long long)blockDim.x + threadIdx.x; base < P;
+       base += U * stride) {
+    float2 v[U][3];
 #pragma unroll
-    for (int a = 0; a < 6; ++a) v[a] = F[(EX + a) * P + i];
-    bool ok = true;
+    for (int r = 0; r < U; ++r) {
+      const long long i = base + r * stride;
 #pragma unroll
-    for (int a = 0; a < 6; ++a) ok &= v[a] == 0.f || df_range(fabsf(v[a]));
-    if (ok) {
-#pragma unroll
-      for (int a = 0; a < 6; ++a) add_to(a < 3 ? e : b, square(v[a]));
-    } else {
-#pragma unroll
-      for (int a = 0; a < 6; ++a) (a < 3 ? se : sb) += (double)v[a] * v[a];
+      for (int a = 0; a < 3; ++a)
+        v[r][a] = i < P ? make_float2(F[(EX + a) * P + i], F[(BX + a) * P + i]) : make_float2(0.f, 0.f);
     }
-    if (++terms == kDfTerms) {
+#pragma unroll
+    for (int r = 0; r < U; ++r) {
+      if (!sum3_range(v[r][0].x, v[r][1].x, v[r][2].x)) {
+        se += squares_fp64(v[r][0].x, v[r][1].x, v[r][2].x);
+        v[r][0].x = v[r][1].x = v[r][2].x = 0.f;  // adds nothing below
+      }
+      if (!sum3_range(v[r][0].y, v[r][1].y, v[r][2].y)) {
+        sb += squares_fp64(v[r][0].y, v[r][1].y, v[r][2].y);
+        v[r][0].y = v[r][1].y = v[r][2].y = 0.f;
+      }
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        float2 p;
+        const float2 l = square(v[r][a], p);
+        sum.add_term(p, l);
+      }
+    }
+    terms += U;
+    if (terms == kSumTerms) {
       terms = 0;
-      se += (double)e.h + e.l;
-      sb += (double)b.h + b.l;
-      e = b = {0.f, 0.f};
+      se += sum.x();
+      sb += sum.y();
+      sum = {};
     }
   }
-  se += (double)e.h + e.l;
-  sb += (double)b.h + b.l;
+  se += sum.x();
+  sb += sum.y();
   se = block_sum(se, sh);
   sb = block_sum(sb, sh);
   if (threadIdx.x == 0) {
-    atomicAdd(&acc[0], 0.5 * se);
-    atomicAdd(&acc[1], 0.5 * sb);
+    atomicAdd(acc, 0.5 * se);
+    atomicAdd(acc + 1, 0.5 * sb);
   }
 }
 
