@@ -36,50 +36,6 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   return s;  // valid in thread 0
 }
 
-// Double-float arithmetic: a value as the unevaluated sum h + l of two floats,
-// |l| <= ulp(h)/2 (Dekker 1971; the error-free sum is Knuth's, the error-free
-// product the fused multiply-add's).  The GPU's FP64 pipe issues one operation
-// for some thirty FP32 ones, so the diagnostics form their terms, 46 to 48
-// bits of them, in FP32 pairs and keep FP64 for the sums over many terms.
-struct DF {
-  float h, l;
-};
-__device__ __forceinline__ DF two_sum(float a, float b) {
-  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
-  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
-}
-__device__ __forceinline__ DF fast_two_sum(float a, float b) {  // |a| >= |b| or a == 0
-  const float s = __fadd_rn(a, b);
-  return {s, __fsub_rn(b, __fsub_rn(s, a))};
-}
-__device__ __forceinline__ DF square(float a) {
-  const float p = __fmul_rn(a, a);
-  return {p, __fmaf_rn(a, a, -p)};
-}
-__device__ __forceinline__ void add_to(DF& s, DF x) {  // s.l collects what s.h rounds off
-  const DF t = two_sum(s.h, x.h);
-  s.h = t.h;
-  s.l = __fadd_rn(s.l, __fadd_rn(t.l, x.l));
-}
-// approximations with a relative error below 2^-22 for normal arguments
-__device__ __forceinline__ float rsqrt_approx(float x) {
-  float r;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-__device__ __forceinline__ float rcp_approx(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-
-// Range of magnitudes whose squares a double-float holds with all its bits.
-constexpr float kDfMin = 9.094947e-13f;   // 2^-40
-constexpr float kDfMax = 1.1529215e18f;   // 2^60
-__device__ __forceinline__ bool df_range(float m) { return m >= kDfMin && m <= kDfMax; }
-
-constexpr int kDfTerms = 16;  // terms summed in double-float before the FP64 sum takes them
-
 // The GPU's FP64 pipe issues one operation for some thirty FP32 ones, so the
 // diagnostics form their terms and the sums of a thread's terms as sums of three
 // floats, s0 + s1 + s2, each about 2^-24 of the one before: 64 bits and more,
@@ -112,6 +68,18 @@ struct Sum3 {
   __device__ __forceinline__ double x() const { return (double)s0.x + ((double)s1.x + s2.x); }
   __device__ __forceinline__ double y() const { return (double)s0.y + ((double)s1.y + s2.y); }
 };
+// approximations with a relative error below 2^-21 for normal arguments
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 // Whether the squares of three floats can be summed this way: the sum of their
 // magnitudes is 0 or between 2^-40 and 2^60 (not for NaN and infinities).
 // Others take FP64.
@@ -122,7 +90,7 @@ __device__ __forceinline__ bool sum3_range(float a, float b, float c) {
 
 constexpr int kSumTerms = 16;  // points or pairs of a thread before its FP64 sum takes them
 
-// not inlined: a branch, not FP64 operations that every thread goes through
+// Not inlined: a branch, not FP64 operations that every thread goes through.
 __device__ __noinline__ double squares_fp64(float a, float b, float c) {
   return (double)a * a + (double)b * b + (double)c * c;
 }
@@ -182,34 +150,50 @@ __global__ void k_field_energy(const float* __restrict__ F, long long P, double*
   }
 }
 
-// gamma - 1 = u^2 / (gamma + 1) in double-float, for max |u_a| in df_range:
-// the squares and their sum without error, gamma and the quotient by one
-// Newton correction each of their FP32 values (relative error below 2^-44).
-__device__ __forceinline__ DF gamma_minus_1(float a, float b, float c) {
-  const DF pa = square(a), pb = square(b), pc = square(c);
-  const DF s1 = two_sum(pa.h, pb.h), s2 = two_sum(s1.h, pc.h);
-  const DF u2 = fast_two_sum(s2.h, ((pa.l + pb.l) + pc.l) + (s1.l + s2.l));
-  const DF x = two_sum(1.0f, u2.h);
-  const float y = rsqrt_approx(x.h), g0 = __fmul_rn(x.h, y);
-  const float g1 = __fmul_rn(__fadd_rn(__fmaf_rn(-g0, g0, x.h), __fadd_rn(x.l, u2.l)), 0.5f * y);
-  const DF d = two_sum(g0, 1.0f);
-  const float r = rcp_approx(d.h), t = __fmul_rn(u2.h, r);
-  const float rem = __fmaf_rn(-t, __fadd_rn(d.l, g1), __fadd_rn(__fmaf_rn(-t, d.h, u2.h), u2.l));
-  return {t, __fmul_rn(rem, r)};
+// t = gamma - 1 as t0 + t1 + t2, for components in sum3_range: the root of
+// t (t + 2) = u^2.  u^2 is held to 2^-68 of its value, t0 is its FP32 value, and
+// t1 and t2 are the corrections that the remainder u^2 - t (t + 2), formed from
+// error-free products and sums, asks for (divided by 2 (t + 1), whose reciprocal
+// is half of 1/gamma): the sum is good to 2^-62.
+__device__ __forceinline__ void gamma_minus_1(float2 a, float2 b, float2 c, float2& t0, float2& t1,
+                                              float2& t2) {
+  float2 pa, pb, pc, s, u0, u1, m, q;
+  const float2 la = square(a, pa), lb = square(b, pb), lc = square(c, pc);
+  const float2 e1 = two_sum(pa, pb, s), e2 = two_sum(s, pc, u0);
+  const float2 f1 = two_sum(e1, e2, m), f2 = two_sum(la, lb, q), f3 = two_sum(q, lc, q),
+               f4 = two_sum(m, q, u1);
+  const float2 u2 = add(add(f1, f2), add(f3, f4));
+  const float2 x = add(u0, make_float2(1.f, 1.f));
+  const float2 y = make_float2(rsqrt_approx(x.x), rsqrt_approx(x.y));
+  const float2 g1 = fma(x, y, make_float2(1.f, 1.f));
+  t0 = mul(u0, make_float2(rcp_approx(g1.x), rcp_approx(g1.y)));
+  const float2 hy = mul(y, make_float2(0.5f, 0.5f)), tt = add(t0, t0);
+  // u^2 - t0^2 - 2 t0: the leading parts agree to 2^-20, their difference is exact
+  float2 p, d, r;
+  const float2 lp = square(t0, p), ld = two_sum(p, tt, d);
+  const float2 h1 = two_sum(add(u0, neg(d)), u1, r), h2 = two_sum(r, neg(ld), r),
+               h3 = two_sum(r, neg(lp), r);
+  const float2 rest = add(add(h1, h2), add(h3, u2));
+  t1 = mul(r, hy);
+  float2 w;  // 2 t0 + 2
+  const float2 lw = two_sum(tt, make_float2(2.f, 2.f), w);
+  const float2 r1 = add(fma(neg(t1), w, r), rest);
+  t2 = mul(fma(neg(t1), add(lw, t1), r1), hy);
 }
 
 // Sum of m c^2 (gamma - 1).  With square root and quotient in FP64 the FP64
-// pipe bounded it, 769 us for 16.8 M particles; with terms in double-float and
-// 16 of them to an FP64 addition it takes 60 us, bound by FP32 issue (the
-// reads alone would take 30 us).
+// pipe bounded it, 769 us for 16.8 M particles; with terms of three floats,
+// two particles to an instruction, it takes 81 us, bound by FP32 arithmetic
+// (some 115 packed operations a pair; the reads alone would take 30 us; terms of
+// two floats, good to 2^-44 only, took 60).
 __global__ void __launch_bounds__(256) k_kinetic(const float* __restrict__ u, long long n,
                                                  long long ld, double mc2, double* acc) {
   __shared__ double sh[32];
   double s = 0.0;
-  DF sum = {0.f, 0.f};
+  Sum3 sum = {};
   int terms = 0;
   const long long stride = (long long)gridDim.x * blockDim.x;
-  constexpr int U = 4;  // rounds whose loads are issued together
+  constexpr int U = 4;  // rounds whose loads are issued together, two to a pair
   for (long long base = blockIdx.x * (long long)blockDim.x + threadIdx.x; base < n;
        base += U * stride) {
     float v[U][3];
@@ -221,25 +205,28 @@ __global__ void __launch_bounds__(256) k_kinetic(const float* __restrict__ u, lo
     }
 #pragma unroll
     for (int r = 0; r < U; ++r) {
-      const float m = fmaxf(fabsf(v[r][0]), fmaxf(fabsf(v[r][1]), fabsf(v[r][2])));
-      const bool at_rest = v[r][0] == 0.f && v[r][1] == 0.f && v[r][2] == 0.f;
-      const bool nan = v[r][0] != v[r][0] || v[r][1] != v[r][1] || v[r][2] != v[r][2];
-      if (df_range(m) && !nan) {
-        add_to(sum, gamma_minus_1(v[r][0], v[r][1], v[r][2]));
-      } else if (!at_rest) {
-        const double a = v[r][0], b = v[r][1], c = v[r][2];
-        const double u2 = a * a + b * b + c * c;
+      if (!sum3_range(v[r][0], v[r][1], v[r][2])) {
+        const double u2 = squares_fp64(v[r][0], v[r][1], v[r][2]);
         s += u2 / (sqrt(1.0 + u2) + 1.0);
+        v[r][0] = v[r][1] = v[r][2] = 0.f;  // adds nothing below
       }
     }
-    terms += U;
-    if (terms == kDfTerms) {
+#pragma unroll
+    for (int r = 0; r < U; r += 2) {
+      float2 t0, t1, t2;
+      gamma_minus_1(make_float2(v[r][0], v[r + 1][0]), make_float2(v[r][1], v[r + 1][1]),
+                    make_float2(v[r][2], v[r + 1][2]), t0, t1, t2);
+      sum.add_term(t0, t1);
+      sum.s2 = add(sum.s2, t2);
+    }
+    terms += U / 2;
+    if (terms == kSumTerms) {
       terms = 0;
-      s += (double)sum.h + sum.l;
-      sum = {0.f, 0.f};
+      s += sum.x() + sum.y();
+      sum = {};
     }
   }
-  s += (double)sum.h + sum.l;
+  s += sum.x() + sum.y();
   s = block_sum(s, sh);
   if (threadIdx.x == 0) atomicAdd(acc, mc2 * s);
 }
