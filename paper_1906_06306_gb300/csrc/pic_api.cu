@@ -267,7 +267,7 @@ std::string derive_tiles(const pic_grid& grid, const pic_tuning& tun, long long 
   if (wcells > (1LL << 24)) return "tile + halo window too large";
   r.wcells = (int)wcells;
   r.wstride = (int)((wcells + 3) / 4 * 4);
-  if ((long long)particle_smem_bytes(grid.dim, r) > 200 * 1024)
+  if (particle_smem_bytes(grid.dim, r, kQueueInLimit) > (size_t)kWindowLimit)
     return "tile + halo window exceeds 200 KB of shared memory";
   if (ntiles > (1LL << 30)) return "too many tiles";
   r.ntiles = (int)ntiles;
@@ -809,7 +809,7 @@ pic_status pic_init(pic_ctx** out, const pic_grid* grid, const pic_species* spec
   }
   pic_status s = PIC_OK;
   cudaError_t e = cudaSuccess;
-  if ((e = set_particle_smem_limit(200 * 1024)) != cudaSuccess) {
+  if ((e = set_particle_smem_limit(kParticleSmem)) != cudaSuccess) {
     s = cuda_fail(nullptr, "cudaFuncSetAttribute", e);
   } else if ((e = dalloc(&ctx->d_status, 1)) != cudaSuccess ||
              (e = cudaMemsetAsync(ctx->d_status, 0, sizeof(int), ctx->st)) != cudaSuccess ||

@@ -130,6 +130,11 @@ constexpr int kSpillEvery = PIC_SPILL_EVERY;
 // end of each species and at a spill point where it is more than half full; a
 // stray that finds it full is processed at once by its own lane.
 constexpr int kQueueCap = 1024;
+// A window is accepted if it fits in this much shared memory with a queue of
+// kQueueInLimit entries; the longer queue's rest comes on top of the limit.
+constexpr int kWindowLimit = 200 * 1024;
+constexpr int kQueueInLimit = 512;
+constexpr int kParticleSmem = kWindowLimit + 4 * (kQueueCap - kQueueInLimit);
 // Particle records of a batch streamed into shared memory by bulk copies
 // (1D/2D fused kernels): a ring of this many stages of kPushThreads records.
 constexpr int kRecStages = 2;
@@ -226,7 +231,7 @@ void set_global_error(const char* msg);
 // crossers are processed by two small kernels after it.
 cudaError_t launch_particles(int dim, int mode, const PushParams& P, cudaStream_t st);
 cudaError_t set_particle_smem_limit(int bytes);
-size_t particle_smem_bytes(int dim, const TileDev& t);
+size_t particle_smem_bytes(int dim, const TileDev& t, int queue = kQueueCap);
 // floats of a block's shared memory past the staged field window, from the
 // first 128-byte boundary on: room for the 2D window's tensor copy
 long long window_landing_floats(int dim, const TileDev& t);

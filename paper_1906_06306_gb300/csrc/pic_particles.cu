@@ -942,13 +942,13 @@ long long window_landing_floats(int dim, const TileDev& t) {
   return (long long)(particle_smem_bytes(dim, t) / sizeof(float)) - field_words(nf, t.wcells) - 31;
 }
 
-size_t particle_smem_bytes(int dim, const TileDev& t) {
+size_t particle_smem_bytes(int dim, const TileDev& t, int queue) {
   const int nf = dim == 1 ? field_floats<1>() : dim == 2 ? field_floats<2>() : field_floats<3>();
   const int jw = (dim == 2 && kJ64<2>) ? 6 : 3;  // int window words per cell
   const int jf = dim == 3 && kFoldGlobal<3> ? 0 : 3;  // float window words per cell
   // 1D/2D: the stray queue and the ring of streamed particle records
   const size_t ring = PIC_TMA_RECORDS ? (size_t)kRecStages * (1 + dim + 3) * kPushThreads : 0;
-  size_t words = (size_t)(jw + jf) * t.wstride + (dim < 3 ? kQueueCap + ring : 0);
+  size_t words = (size_t)(jw + jf) * t.wstride + (dim < 3 ? queue + ring : 0);
   // 2D: the same area first takes the window's tensor copy, E and B over a box
   // whose x extent is the window's widened to 16-byte ends, after up to 31
   // floats of padding to a 128-byte boundary

@@ -1,0 +1,35 @@
+"""The largest tile windows that pic_set_tuning accepts: 200 KB of shared memory
+with a stray queue of 512 entries (the queue is longer)."""
+import numpy as np
+import pytest
+
+import workloads
+from gpu_helpers import compare_fields, oracle_from_sim, step_floor
+
+pytestmark = pytest.mark.gpu
+
+# (dim, box, largest accepted tile, halo, the next larger one): 14 words a window cell in
+# 1D, 12 in 2D, and 512 words, in 51,200
+WINDOWS = [(1, (4000, 1, 1), (3613, 1, 1), 3, (3614, 1, 1)),
+           (2, (90, 100, 1), (55, 57, 1), 4, (56, 57, 1))]
+
+
+@pytest.mark.parametrize("dim,n,tile,halo,larger", WINDOWS)
+def test_largest_window_is_accepted_and_steps(dim, n, tile, halo, larger):
+    import oracle
+    from paper_1906_06306_gb300 import Simulation
+    from paper_1906_06306_gb300 import binding as B
+
+    pl = workloads.uniform_plasma(dim, *n, 0.45, 6, 0.01, 0.5, seed=11)
+    sim = Simulation.from_plasma(pl)
+    with pytest.raises(B.PicError):
+        sim.set_tuning(tile=larger, halo=halo)
+    sim.set_tuning(tile=tile, halo=halo, sort_every=1000)
+    sim.sort()
+    g, F, osp, _ = oracle_from_sim(sim)
+    floor = step_floor(g, osp, 2)
+    sim.step(2)
+    sim.check()
+    oracle.step(g, F, osp, nsteps=2)
+    compare_fields(sim.download()[0], F, floor=floor)
+    sim.close()
