@@ -576,12 +576,13 @@ __global__ void __launch_bounds__(256, D == 3 ? 2 : PIC_ADJ_MIN_BLOCKS)
     int a, b;
     adj_share(P, S, B, a, b);
     const long long ld = S.ld;
-    for (int base = a; base < b; base += blockDim.x) {  // the same count for every thread
-      const int p = base + threadIdx.x;
+    // the same count of batches for every thread
+    for (SlotWalk walk = slot_walk(a, b, blockDim.x, false, false); walk.more(); walk.next(blockDim.x)) {
+      const slot_t p = walk.slot(threadIdx.x);
       float ebb[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, o[3] = {0.f, 0.f, 0.f}, xb[3];
       int l[3] = {0, 0, 0};
       bool mine = false;
-      if (p < b) {
+      if (walk.mine(p)) {
         const int cell = S.cell[p];
         if (cell >= 0 && (long long)cell < plane) {
           if (adj_in_window<D>(P, B, cell, l)) {

@@ -10,6 +10,8 @@
 
 #include <type_traits>
 
+#include "pic_slots.h"
+
 namespace pic {
 
 enum { EX = 0, EY, EZ, BX, BY, BZ, JX, JY, JZ };
