@@ -516,22 +516,22 @@ __global__ void __launch_bounds__(kPushThreads, D == 3 ? PIC_PUSH_MIN_BLOCKS_3D
   // the next batch to issue; pr_s == nspecies when everything is issued
   // (in shared memory: only thread 0 uses it, and registers are scarce)
   __shared__ struct {
-    int s, base;  // species and first index of the next batch to issue (s == nspecies: done)
+    int s;        // species of the next batch to issue (nspecies: done)
+    slot_t base;  // its first index
     int issued;   // batches issued
     int seen;     // batches thread 0 found complete
   } pr;
   auto pr_next_species = [&](int s) {
     while (s < P.nspecies && rng_a[s] >= rng_b[s]) ++s;
     pr.s = s;
-    if (s < P.nspecies) pr.base = rng_a[s] & ~3;
+    if (s < P.nspecies) pr.base = (slot_t)rng_a[s] & ~3u;
   };
   // issue batch j (the producer's next) into stage j % kRecStages
   auto pr_issue = [&](int j) {
     const SpeciesDev& S = P.sp[pr.s];
-    const int base = pr.base;
-    const int end4 = (rng_b[pr.s] + 3) & ~3;
-    const int cnt = end4 - base < kPushThreads ? end4 - base : kPushThreads;
-    const unsigned bytes = 4u * (unsigned)cnt;
+    const slot_t base = pr.base, end4 = ((slot_t)rng_b[pr.s] + 3u) & ~3u;
+    const slot_t cnt = end4 - base < kPushThreads ? end4 - base : kPushThreads;
+    const unsigned bytes = 4u * cnt;
     unsigned long long* bar = &bar_full[j % kRecStages];
     float* dst = ring + (j % kRecStages) * NR * kPushThreads;
     mbar_arrive_expect_tx(bar, bytes * NR);
@@ -543,7 +543,7 @@ __global__ void __launch_bounds__(kPushThreads, D == 3 ? PIC_PUSH_MIN_BLOCKS_3D
       bulk_load(dst + (1 + D + a) * kPushThreads, S.ru + a * S.ld + base, bytes, bar);
     pr.issued = j + 1;
     pr.base = base + kPushThreads;
-    if (pr.base >= rng_b[pr.s]) pr_next_species(pr.s + 1);
+    if (pr.base >= (slot_t)rng_b[pr.s]) pr_next_species(pr.s + 1);
   };
   bool dead = false;  // this thread gave up on the stream after a timed-out wait
 
@@ -791,13 +791,10 @@ __global__ void __launch_bounds__(kPushThreads, D == 3 ? PIC_PUSH_MIN_BLOCKS_3D
     if (PIC_PREFETCH && !TMA && a + (int)threadIdx.x < b) load_rec<D, MODE>(S, a + threadIdx.x, cur);
     // block-uniform trip count; with the stream the batches start 16-byte aligned,
     // in 3D on a 128-byte line (kLineBatches)
-    int base = TMA && a < b ? a & ~3 : a;
-    if (kLineBatches<D, MODE> && !TMA && !PIC_PREFETCH &&
-        (b - a + kPushThreads - 1) / kPushThreads == (b - (a & ~31) + kPushThreads - 1) / kPushThreads)
-      base = a & ~31;
-    for (; base < b; base += blockDim.x) {
-      const int p = base + threadIdx.x;
-      bool in = p >= a && p < b;
+    for (SlotWalk walk = slot_walk(a, b, kPushThreads, kLineBatches<D, MODE> && !TMA && !PIC_PREFETCH, TMA);
+         walk.more(); walk.next(blockDim.x)) {
+      const slot_t p = walk.slot(threadIdx.x);
+      bool in = walk.mine(p);
       if (TMA) {
         const int stage = kk % kRecStages;
         if (!dead) {
@@ -830,7 +827,7 @@ __global__ void __launch_bounds__(kPushThreads, D == 3 ? PIC_PUSH_MIN_BLOCKS_3D
         }
         ++kk;
       } else if (PIC_PREFETCH) {
-        if (p + (int)blockDim.x < b) load_rec<D, MODE>(S, p + blockDim.x, nxt);
+        if (walk.mine(p + blockDim.x)) load_rec<D, MODE>(S, p + blockDim.x, nxt);
       } else if (in) {
         load_rec<D, MODE>(S, p, cur);
       }
@@ -927,7 +924,7 @@ __global__ void __launch_bounds__(kPushThreads) k_particles_deferred(const PushP
   for (int s = 0; s < P.nspecies; ++s) {
     const SpeciesDev& S = P.sp[s];
     const int cnt = *S.dcount;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x) {
+    for (slot_t i = blockIdx.x * blockDim.x + threadIdx.x; i < (slot_t)cnt; i += gridDim.x * blockDim.x) {
       const int p = S.dlist[i];
       PRec r;
       load_rec<D, MODE>(S, p, r);
