@@ -356,16 +356,16 @@ __device__ __forceinline__ float rcp_from_1(float x) {
 // (Markstein, "Computation of elementary functions on the IBM RISC System/6000",
 // 1990), which leaves out the range tests that the general routines carry.  For
 // every float in [1, inf) the result is that of __frcp_rn(__fsqrt_rn(x))
-// (compared one by one); x = inf gives 0 as those do.  With the two
-// approximations above: 1024^2 turbulence 5942 -> 5836 us per 10 steps, 3D
-// shock-shaped run 14725 -> 14564 per 3 (the kernels are issue bound).
+// (compared one by one); x = inf gives 0 and NaN gives NaN as those do.  With
+// the two approximations above: 1024^2 turbulence 5942 -> 5836 us per 10 steps,
+// 3D shock-shaped run 14725 -> 14564 per 3 (the kernels are issue bound).
 __device__ __forceinline__ float inverse_sqrt_rn(float x) {
   const float y = rsqrt_from_1(x);
   const float s0 = __fmul_rn(x, y);
   const float s = __fmaf_rn(__fmaf_rn(-s0, s0, x), __fmul_rn(0.5f, y), s0);
   const float r0 = rcp_from_1(s);
   const float r = __fmaf_rn(__fmaf_rn(-s, r0, 1.0f), r0, r0);
-  return x < __int_as_float(0x7f800000) ? r : 0.0f;
+  return x == __int_as_float(0x7f800000) ? 0.0f : r;
 }
 
 // Relativistic Boris scheme, Appendix C: u1 = c u + (s/2) E,
