@@ -1205,10 +1205,10 @@ pic_status pic_field_update(pic_ctx* ctx, int which) {
 }
 
 // The conducting wall's field condition after a field update (shock boxes).
-cudaError_t wall_fields(pic_ctx* ctx) {
+cudaError_t wall_fields(pic_ctx* ctx, int push_next = 0) {
   if (!ctx->shock) return cudaSuccess;
   return timed(ctx, PIC_KERNEL_BOUNDARY, [&]() {
-    return launch_wall_fields(ctx->g, ctx->F, ctx->wall, ctx->i_zero, ctx->st);
+    return launch_wall_fields(ctx->g, ctx->F, ctx->wall, ctx->i_zero, ctx->st, push_next);
   });
 }
 
@@ -1267,7 +1267,6 @@ pic_status pic_step(pic_ctx* ctx, int nsteps) {
     ctx->snapshot_valid = false;
     nsteps -= full * cyc;
   }
-  const auto wall_bc = [&]() { return wall_fields(ctx); };
   bool b1_done = false;  // this step's first B half step ran with the last field launch
   for (int it = 0; it < nsteps; ++it) {
     InjectParams IP{};
@@ -1290,8 +1289,9 @@ pic_status pic_step(pic_ctx* ctx, int nsteps) {
     ctx->sorted_pending = false;
     cudaError_t e = cudaSuccess;
     if (!b1_done) {
-      e = timed(ctx, PIC_KERNEL_BHALF, [&]() { return launch_b_half(ctx->g, ctx->F, 1, ctx->st); });
-      if (e == cudaSuccess) e = wall_bc();
+      e = timed(ctx, PIC_KERNEL_BHALF,
+                [&]() { return launch_b_half(ctx->g, ctx->F, 1, ctx->st, !ctx->shock); });
+      if (e == cudaSuccess) e = wall_fields(ctx, 1);
       if (e != cudaSuccess) return cuda_fail(ctx, "B half step", e);
     }
     e = timed(ctx, PIC_KERNEL_PUSH, [&]() { return launch_particles(ctx->grid.dim, 0, P, ctx->st); });
@@ -1490,7 +1490,7 @@ pic_status step_host_copies(pic_ctx* ctx, const pic_host_species* hs, float* hos
   if (sort) sort_done(ctx, false);
   const PushParams P = make_params(ctx);
   ctx->sorted_pending = false;
-  cudaError_t e = launch_b_half(ctx->g, ctx->F, 1, ctx->st);
+  cudaError_t e = launch_b_half(ctx->g, ctx->F, 1, ctx->st, 1);
   if (e != cudaSuccess) return cuda_fail(ctx, "B half step", e);
   for (int s = 0; s < ns; ++s) {
     if (sort) {  // the count covers the whole species

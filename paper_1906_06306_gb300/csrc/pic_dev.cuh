@@ -110,9 +110,18 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned b
 // stream is complete and its writes are visible, then let the next one be set
 // up.  In this order: once a kernel runs, all but the one before it are
 // complete.
-__device__ __forceinline__ void grid_dependency() {
+// Not before the particle kernel (push_next): its blocks, placed while some SMs
+// still hold a field kernel's, are spread unevenly, and where they all run in
+// one wave the fullest SM decides.  It is set up when the field kernel's blocks
+// have exited, which still hides its launch.  Microseconds a step of 2D boxes,
+// in a run of 20 and alone, with early set-up | without programmatic launch |
+// like this: 96^2 cells x 24 particles (432 blocks) 21.4 | 18.8 | 18.7 and 21.3 |
+// 21.7 | 19.0; 128^2 x 32 (576) 28.3 | 25.9 | 25.8 and 30.3 | 29.7 | 27.5; 256^2 x
+// 16 (512) 45.4 | 40.3 | 40.3 and 49.8 | 44.3 | 42.0; 512^2 x 32 (2048, more than
+// a wave) 181 in all three and 187 | 189 | 185.
+__device__ __forceinline__ void grid_dependency(int push_next = 0) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (!push_next) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 struct GridDev {

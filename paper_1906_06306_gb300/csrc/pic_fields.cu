@@ -45,8 +45,9 @@ __device__ __forceinline__ void b_half_point(float* __restrict__ F, const GridDe
 }
 
 template <int D>
-__global__ void k_b_half(float* __restrict__ F, const GridDev g, float hc, int zero_j) {
-  grid_dependency();
+__global__ void k_b_half(float* __restrict__ F, const GridDev g, float hc, int zero_j,
+                         int push_next) {
+  grid_dependency(push_next);
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n0) return;
@@ -158,8 +159,9 @@ __device__ __forceinline__ void arr4(const float4 a, float v[4]) {
 }
 
 template <int D>
-__global__ void k_b_half_x4(float* __restrict__ F, const GridDev g, float hc, int zero_j) {
-  grid_dependency();
+__global__ void k_b_half_x4(float* __restrict__ F, const GridDev g, float hc, int zero_j,
+                            int push_next) {
+  grid_dependency(push_next);
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
   const long long P = g.plane;
   const int i = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
@@ -333,8 +335,9 @@ __device__ __forceinline__ float d4m(const float* A, long long i, const Nb& b) {
 
 // FDTD4 versions of the two updates (same structure as above, wider stencil).
 template <int D>
-__global__ void k_b_half4(float* __restrict__ F, const GridDev g, float hc, int zero_j) {
-  grid_dependency();
+__global__ void k_b_half4(float* __restrict__ F, const GridDev g, float hc, int zero_j,
+                          int push_next) {
+  grid_dependency(push_next);
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
   const long long P = g.plane;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -417,26 +420,26 @@ static RowLaunch row_launch_x4(const GridDev& g) {
   return row_launch(q);
 }
 
-cudaError_t launch_b_half(const GridDev& g, float* F, int zero_j, cudaStream_t st) {
+cudaError_t launch_b_half(const GridDev& g, float* F, int zero_j, cudaStream_t st, int push_next) {
   const float hc = 0.5f * g.c;
   if (g.order == 2 && x4_ok(g, F)) {
     const RowLaunch L = row_launch_x4(g);
     switch (g.dim) {
-      case 1: launch_kernel(g.pdl, k_b_half_x4<1>, L.grid, L.threads, 0, st, F, g, hc, zero_j); break;
-      case 2: launch_kernel(g.pdl, k_b_half_x4<2>, L.grid, L.threads, 0, st, F, g, hc, zero_j); break;
-      case 3: launch_kernel(g.pdl, k_b_half_x4<3>, L.grid, L.threads, 0, st, F, g, hc, zero_j); break;
+      case 1: launch_kernel(g.pdl, k_b_half_x4<1>, L.grid, L.threads, 0, st, F, g, hc, zero_j, push_next); break;
+      case 2: launch_kernel(g.pdl, k_b_half_x4<2>, L.grid, L.threads, 0, st, F, g, hc, zero_j, push_next); break;
+      case 3: launch_kernel(g.pdl, k_b_half_x4<3>, L.grid, L.threads, 0, st, F, g, hc, zero_j, push_next); break;
       default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
   }
   const RowLaunch L = row_launch(g);
   switch (g.dim * 10 + g.order) {
-    case 12: launch_kernel(g.pdl, k_b_half<1>, L.grid, L.threads, 0, st, F, g, hc, zero_j); break;
-    case 22: launch_kernel(g.pdl, k_b_half<2>, L.grid, L.threads, 0, st, F, g, hc, zero_j); break;
-    case 32: launch_kernel(g.pdl, k_b_half<3>, L.grid, L.threads, 0, st, F, g, hc, zero_j); break;
-    case 14: launch_kernel(g.pdl, k_b_half4<1>, L.grid, L.threads, 0, st, F, g, hc, zero_j); break;
-    case 24: launch_kernel(g.pdl, k_b_half4<2>, L.grid, L.threads, 0, st, F, g, hc, zero_j); break;
-    case 34: launch_kernel(g.pdl, k_b_half4<3>, L.grid, L.threads, 0, st, F, g, hc, zero_j); break;
+    case 12: launch_kernel(g.pdl, k_b_half<1>, L.grid, L.threads, 0, st, F, g, hc, zero_j, push_next); break;
+    case 22: launch_kernel(g.pdl, k_b_half<2>, L.grid, L.threads, 0, st, F, g, hc, zero_j, push_next); break;
+    case 32: launch_kernel(g.pdl, k_b_half<3>, L.grid, L.threads, 0, st, F, g, hc, zero_j, push_next); break;
+    case 14: launch_kernel(g.pdl, k_b_half4<1>, L.grid, L.threads, 0, st, F, g, hc, zero_j, push_next); break;
+    case 24: launch_kernel(g.pdl, k_b_half4<2>, L.grid, L.threads, 0, st, F, g, hc, zero_j, push_next); break;
+    case 34: launch_kernel(g.pdl, k_b_half4<3>, L.grid, L.threads, 0, st, F, g, hc, zero_j, push_next); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

@@ -236,7 +236,9 @@ size_t particle_smem_bytes(int dim, const TileDev& t, int queue = kQueueCap);
 // first 128-byte boundary on: room for the 2D window's tensor copy
 long long window_landing_floats(int dim, const TileDev& t);
 
-cudaError_t launch_b_half(const GridDev& g, float* F, int zero_j, cudaStream_t st);
+// push_next: the particle kernel is launched next (grid_dependency)
+cudaError_t launch_b_half(const GridDev& g, float* F, int zero_j, cudaStream_t st,
+                          int push_next = 0);
 // J: the three current planes, F's own or the filter's buffer (then also
 // copied to F's)
 cudaError_t launch_e_update(const GridDev& g, float* F, const float* J, cudaStream_t st);
@@ -334,7 +336,8 @@ cudaError_t launch_gauss(const GridDev& g, const float* F, const double* rho, in
 // Shock boundaries (Sect. 4.2): the conducting wall's field boundary (zero
 // tangential E on the node plane x = wall, mirror image behind it) and zero E
 // and B at i >= i_zero, applied after each field update.
-cudaError_t launch_wall_fields(const GridDev& g, float* F, int wall, int i_zero, cudaStream_t st);
+cudaError_t launch_wall_fields(const GridDev& g, float* F, int wall, int i_zero, cudaStream_t st,
+                               int push_next = 0);
 
 // One contiguous run of injected particles: template indices [k0, k1) of copy
 // m of species s, written from output index `out` on, x = x_t + shift.

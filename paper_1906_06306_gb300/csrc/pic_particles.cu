@@ -1013,16 +1013,6 @@ cudaError_t set_particle_smem_limit(int bytes) {
 template <int D, int MODE>
 static cudaError_t launch(const PushParams& P, cudaStream_t st) {
   const unsigned nblocks = (unsigned)P.t.ntiles * (unsigned)P.splits;
-  // Blocks placed while the last kernel's are still on the SMs are spread less
-  // evenly.  Where all blocks run in one wave and are long (from 2048 particles
-  // on) the fullest SM decides, and that costs more than the early set-up
-  // gains: 133^2 box, 648 blocks of 2184 particles, 20 steps 1055 us with,
-  // 1008 without; 130 x 94 box, 648 blocks of 300, a step 29.0 with, 31.3
-  // without; 128^2 box, 640 blocks of 1640, gradient 5.45 ms with, 5.55 without.
-  long long ntot = 0;
-  for (int s = 0; s < P.nspecies; ++s) ntot += P.sp[s].n;
-  const unsigned wave = 152u * (D == 3 ? PIC_PUSH_MIN_BLOCKS_3D : PIC_PUSH_MIN_BLOCKS);
-  const int pdl = P.g.pdl && !(nblocks <= wave && ntot >= 2048LL * nblocks);
   // the deferred lists can have entries in 3D (strays) and with the wall
   constexpr bool deferred = D == 3 || MODE == 3;
   if (deferred) {
@@ -1040,27 +1030,27 @@ static cudaError_t launch(const PushParams& P, cudaStream_t st) {
   constexpr bool kStreamable = PIC_TMA_RECORDS && D < 3 && (MODE == 0 || MODE == 3);
   const bool tma = kStreamable && P.rec_aligned;
   if (D == 2 && MODE == 0 && P.t.W[0] == 23 && P.t.W[1] == 15 && tma)
-    launch_kernel(pdl, k_particles<2, 0, 23, 15, 1, kStreamable>, nblocks, kPushThreads, smem, st, P);
+    launch_kernel(P.g.pdl, k_particles<2, 0, 23, 15, 1, kStreamable>, nblocks, kPushThreads, smem, st, P);
   else if (D == 2 && MODE == 0 && P.t.W[0] == 23 && P.t.W[1] == 23 && tma)
-    launch_kernel(pdl, k_particles<2, 0, 23, 23, 1, kStreamable>, nblocks, kPushThreads, smem, st, P);
+    launch_kernel(P.g.pdl, k_particles<2, 0, 23, 23, 1, kStreamable>, nblocks, kPushThreads, smem, st, P);
   else if (D == 2 && MODE == 0 && P.t.W[0] == 23 && P.t.W[1] == 15)
-    launch_kernel(pdl, k_particles<2, 0, 23, 15>, nblocks, kPushThreads, smem, st, P);
+    launch_kernel(P.g.pdl, k_particles<2, 0, 23, 15>, nblocks, kPushThreads, smem, st, P);
   else if (D == 2 && MODE == 0 && P.t.W[0] == 23 && P.t.W[1] == 23)
-    launch_kernel(pdl, k_particles<2, 0, 23, 23>, nblocks, kPushThreads, smem, st, P);
+    launch_kernel(P.g.pdl, k_particles<2, 0, 23, 23>, nblocks, kPushThreads, smem, st, P);
   else if (D == 2 && MODE == 0 && P.t.W[0] == 25 && P.t.W[1] == 17)
-    launch_kernel(pdl, k_particles<2, 0, 25, 17>, nblocks, kPushThreads, smem, st, P);
+    launch_kernel(P.g.pdl, k_particles<2, 0, 25, 17>, nblocks, kPushThreads, smem, st, P);
   else if (tma)
-    launch_kernel(pdl, k_particles<D, MODE, 0, 0, 1, kStreamable>, nblocks, kPushThreads, smem, st, P);
+    launch_kernel(P.g.pdl, k_particles<D, MODE, 0, 0, 1, kStreamable>, nblocks, kPushThreads, smem, st, P);
   else if (D == 3 && MODE == 0 && w3)
-    launch_kernel(pdl, k_particles<3, 0, 13, 13, 9>, nblocks, kPushThreads, smem, st, P);
+    launch_kernel(P.g.pdl, k_particles<3, 0, 13, 13, 9>, nblocks, kPushThreads, smem, st, P);
   else if (D == 3 && MODE == 3 && w3)
-    launch_kernel(pdl, k_particles<3, 3, 13, 13, 9>, nblocks, kPushThreads, smem, st, P);
+    launch_kernel(P.g.pdl, k_particles<3, 3, 13, 13, 9>, nblocks, kPushThreads, smem, st, P);
   else if (D == 3 && MODE == 0 && w37)
-    launch_kernel(pdl, k_particles<3, 0, 13, 13, 7>, nblocks, kPushThreads, smem, st, P);
+    launch_kernel(P.g.pdl, k_particles<3, 0, 13, 13, 7>, nblocks, kPushThreads, smem, st, P);
   else if (D == 3 && MODE == 3 && w37)
-    launch_kernel(pdl, k_particles<3, 3, 13, 13, 7>, nblocks, kPushThreads, smem, st, P);
+    launch_kernel(P.g.pdl, k_particles<3, 3, 13, 13, 7>, nblocks, kPushThreads, smem, st, P);
   else
-    launch_kernel(pdl, k_particles<D, MODE>, nblocks, kPushThreads, smem, st, P);
+    launch_kernel(P.g.pdl, k_particles<D, MODE>, nblocks, kPushThreads, smem, st, P);
   if ((MODE == 0 || MODE == 3) && P.tail_blocks > 0)
     launch_kernel(P.g.pdl, k_particles_tail<D>, (unsigned)P.tail_blocks, kPushThreads, 0, st, P);
   if (deferred) launch_kernel(P.g.pdl, k_particles_deferred<D, MODE>, 4 * 152, kPushThreads, 0, st, P);

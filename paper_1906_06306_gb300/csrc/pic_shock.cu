@@ -22,8 +22,9 @@ static unsigned grid_for(long long n, int threads) {
 // B at i >= i_zero are zeroed.  The sources 2w - i > w and 2w - 1 - i >= w
 // lie below i_zero (2w < i_zero) and are never written here, so the threads
 // do not race.
-__global__ void k_wall_fields(float* __restrict__ F, const GridDev g, int w, int i_zero) {
-  grid_dependency();
+__global__ void k_wall_fields(float* __restrict__ F, const GridDev g, int w, int i_zero,
+                              int push_next) {
+  grid_dependency(push_next);
   const int n0 = g.n[0];
   const long long P = g.plane;
   const int cols = w + 1 + (n0 - i_zero);
@@ -52,9 +53,11 @@ __global__ void k_wall_fields(float* __restrict__ F, const GridDev g, int w, int
   }
 }
 
-cudaError_t launch_wall_fields(const GridDev& g, float* F, int wall, int i_zero, cudaStream_t st) {
+cudaError_t launch_wall_fields(const GridDev& g, float* F, int wall, int i_zero, cudaStream_t st,
+                               int push_next) {
   const long long work = (g.plane / g.n[0]) * (long long)(wall + 1 + (g.n[0] - i_zero));
-  launch_kernel(g.pdl, k_wall_fields, grid_for(work, 256), 256, 0, st, F, g, wall, i_zero);
+  launch_kernel(g.pdl, k_wall_fields, grid_for(work, 256), 256, 0, st, F, g, wall, i_zero,
+                push_next);
   return cudaGetLastError();
 }
 
