@@ -251,6 +251,18 @@ __global__ void k_tile_scatter_lanes(const SortParams P, const SortSet Q) {
   }
 }
 
+// Whether a warp's particles are of one bin (lanes without one count as of it;
+// lane 0 has one unless none has), or of no more than two, those of its lanes 0
+// and 31.  Every lane of the warp calls these.
+__device__ __forceinline__ bool one_bin(int key, bool active) {
+  const int first = __shfl_sync(0xffffffffu, key, 0);
+  return __all_sync(0xffffffffu, !active || key == first);
+}
+__device__ __forceinline__ bool two_bins(int key, bool active) {
+  const int first = __shfl_sync(0xffffffffu, key, 0), last = __shfl_sync(0xffffffffu, key, 31);
+  return __all_sync(0xffffffffu, !active || key == first || key == last);
+}
+
 // The scatter of many particles.  A block takes U * 256 consecutive ones, puts
 // them into bin order in shared memory and writes each bin's to consecutive
 // slots: the array was sorted some steps ago, so a chunk holds a few bins and
@@ -261,7 +273,15 @@ __global__ void k_tile_scatter_lanes(const SortParams P, const SortSet Q) {
 // block are counted in a table as in k_tile_count, each lane with its own
 // shared atomic, whose result is the particle's place in its bin (combining a
 // warp's equal bins first took 202 us); a particle whose table slot another
-// bin holds reserves its place in the global cursor by itself.
+// bin holds reserves its place in the global cursor by itself.  Lanes of one
+// bin take their places one after the other, which costs most in an array that
+// is in order already.  A warp whose first and last 256th of the chunk show one
+// (no more than two bins each) therefore adds 32 at once where a round's
+// particles are of one bin.  pic_sort on an array in order, two species of
+// 16.8 M: 3D 975 -> 890 us, 2D 731 -> 688; on one in cell order, 2D 883 -> 770;
+// drifted arrays and sorts in a run within 0.3 % (with the look in every round
+// instead, 5 to 10 % more).  Scattered lane by lane, as few particles are below,
+// an array in order takes 800 and 706, a drifted one twice as long as here.
 template <int D, int U>
 __global__ void __launch_bounds__(256) k_tile_scatter(const SortParams P, const SortSet Q) {
   grid_dependency();
@@ -284,27 +304,52 @@ __global__ void __launch_bounds__(256) k_tile_scatter(const SortParams P, const 
   int c[U], slot[U], rank[U];  // slot < 0: no table slot, rank is the place among the lone ones
 #pragma unroll
   for (int r = 0; r < U; ++r) c[r] = r * 256 + t < here ? cell[base + r * 256 + t] : 0;
-  __syncthreads();
   int lone_dst[U];
+  const auto take = [&](int r, int key, int number) {  // this lane's table slot and place, for `number`
+    const int s = (int)(((unsigned)key * 2654435761u) >> 22);  // multiplicative hash, 10 bits
+    int old = *(volatile int*)&skey[s];
+    if (old == -1) old = atomicCAS(&skey[s], -1, key);
+    if (old == -1 || old == key) {
+      slot[r] = s;
+      rank[r] = atomicAdd(&scnt[s], number);
+    } else {
+      slot[r] = -1;
+      rank[r] = atomicAdd(&lone, number);
+      lone_dst[r] = atomicAdd(&cursor[key], number);
+    }
+  };
 #pragma unroll
   for (int r = 0; r < U; ++r) {
     slot[r] = 0;
     rank[r] = 0;
     lone_dst[r] = 0;
-    if (r * 256 + t < here) {
-      const int key = tile_key<D>(P, c[r]);
-      const int s = (int)(((unsigned)key * 2654435761u) >> 22);  // multiplicative hash, 10 bits
-      int old = *(volatile int*)&skey[s];
-      if (old == -1) old = atomicCAS(&skey[s], -1, key);
-      if (old == -1 || old == key) {
-        slot[r] = s;
-        rank[r] = atomicAdd(&scnt[s], 1);
-      } else {
-        slot[r] = -1;
-        rank[r] = atomicAdd(&lone, 1);
-        lone_dst[r] = atomicAdd(&cursor[key], 1);
+  }
+  __syncthreads();
+  const bool in0 = t < here, in1 = (U - 1) * 256 + t < here;
+  if (two_bins(in0 ? tile_key<D>(P, c[0]) : -1, in0) &&
+      two_bins(in1 ? tile_key<D>(P, c[U - 1]) : -1, in1)) {
+    unsigned together = 0;  // bit r: round r's particles of this warp are of one bin
+#pragma unroll
+    for (int r = 0; r < U; ++r) {
+      const bool in = r * 256 + t < here;
+      const int key = in ? tile_key<D>(P, c[r]) : -1;
+      const bool one = one_bin(key, in);
+      if (one) together |= 1u << r;
+      if (in && (!one || lane == 0)) take(r, key, one ? min(32, here - (r * 256 + t)) : 1);
+    }
+    // after the loop, so that its atomics are in flight together
+#pragma unroll
+    for (int r = 0; r < U; ++r) {
+      if (together >> r & 1) {
+        slot[r] = __shfl_sync(0xffffffffu, slot[r], 0);
+        rank[r] = __shfl_sync(0xffffffffu, rank[r], 0) + lane;
+        lone_dst[r] = __shfl_sync(0xffffffffu, lone_dst[r], 0) + lane;
       }
     }
+  } else {
+#pragma unroll
+    for (int r = 0; r < U; ++r)
+      if (r * 256 + t < here) take(r, tile_key<D>(P, c[r]), 1);
   }
   __syncthreads();
   // exclusive scan of the table's counts, 4 slots to a thread; each bin's place
