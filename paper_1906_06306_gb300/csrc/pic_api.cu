@@ -202,6 +202,15 @@ int device_sms() {
   return sms;
 }
 
+// Blocks of the particle kernel that an SM holds: the registers are for
+// PIC_PUSH_MIN_BLOCKS, shared memory may be for fewer (of 228 KB; 1 KB a block is
+// the system's, and some 200 bytes are the kernel's static ones).
+int resident_blocks(int dim, const TileDev& t) {
+  const int by_regs = dim == 3 ? PIC_PUSH_MIN_BLOCKS_3D : PIC_PUSH_MIN_BLOCKS;
+  const int by_smem = (int)(228 * 1024 / (particle_smem_bytes(dim, t) + 1024 + 256));
+  return std::max(1, std::min(by_regs, by_smem));
+}
+
 // Blocks per tile for a box whose particle launch fits the GPU at once: the
 // SMs with the most blocks decide its time, so the blocks should fill a whole
 // number of them per SM.  The estimate for s blocks per tile, in particles of an SM's
@@ -267,8 +276,14 @@ std::string derive_tiles(const pic_grid& grid, const pic_tuning& tun, long long 
   if (wcells > (1LL << 24)) return "tile + halo window too large";
   r.wcells = (int)wcells;
   r.wstride = (int)((wcells + 3) / 4 * 4);
-  if (particle_smem_bytes(grid.dim, r, kQueueInLimit) > (size_t)kWindowLimit)
+  r.queue = kQueueShort;
+  if (particle_smem_bytes(grid.dim, r) > (size_t)kParticleSmem)
     return "tile + halo window exceeds 200 KB of shared memory";
+  TileDev q = r;
+  q.queue = kQueueLong;
+  if (particle_smem_bytes(grid.dim, q) <= (size_t)kParticleSmem &&
+      resident_blocks(grid.dim, q) == resident_blocks(grid.dim, r))
+    r = q;
   if (ntiles > (1LL << 30)) return "too many tiles";
   r.ntiles = (int)ntiles;
   r.nsub = r.ns[0] * r.ns[1] * r.ns[2];

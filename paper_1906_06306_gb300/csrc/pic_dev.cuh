@@ -144,6 +144,7 @@ struct TileDev {
   int S[3];     // sub-tile extents: the sort orders a tile's particles by sub-tile
   int ns[3];    // sub-tiles per tile along each axis
   int nsub;     // sub-tiles per tile (sort bins per tile)
+  int queue;    // entries of the particle kernel's stray queue (1D/2D)
 };
 
 struct SpeciesDev {

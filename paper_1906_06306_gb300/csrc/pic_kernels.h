@@ -128,13 +128,11 @@ constexpr int kSpillEvery = PIC_SPILL_EVERY;
 // Shared-memory queue of the 1D/2D tile kernels for particles outside the tile
 // window (about 0.5 % of the particles between sorts).  It is drained at the
 // end of each species and at a spill point where it is more than half full; a
-// stray that finds it full is processed at once by its own lane.
-constexpr int kQueueCap = 1024;
-// A window is accepted if it fits in this much shared memory with a queue of
-// kQueueInLimit entries; the longer queue's rest comes on top of the limit.
-constexpr int kWindowLimit = 200 * 1024;
-constexpr int kQueueInLimit = 512;
-constexpr int kParticleSmem = kWindowLimit + 4 * (kQueueCap - kQueueInLimit);
+// stray that finds it full is processed at once by its own lane.  The longer
+// queue is for the batches between two folds; a window whose blocks would then
+// be fewer on an SM, or exceed the limit on its shared memory, takes the shorter.
+constexpr int kQueueLong = 1024, kQueueShort = 512;
+constexpr int kParticleSmem = 200 * 1024;
 // Particle records of a batch streamed into shared memory by bulk copies
 // (1D/2D fused kernels): a ring of this many stages of kPushThreads records.
 constexpr int kRecStages = 2;
@@ -231,7 +229,7 @@ void set_global_error(const char* msg);
 // crossers are processed by two small kernels after it.
 cudaError_t launch_particles(int dim, int mode, const PushParams& P, cudaStream_t st);
 cudaError_t set_particle_smem_limit(int bytes);
-size_t particle_smem_bytes(int dim, const TileDev& t, int queue = kQueueCap);
+size_t particle_smem_bytes(int dim, const TileDev& t);
 // floats of a block's shared memory past the staged field window, from the
 // first 128-byte boundary on: room for the 2D window's tensor copy
 long long window_landing_floats(int dim, const TileDev& t);

@@ -482,7 +482,7 @@ __global__ void __launch_bounds__(kPushThreads, D == 3 ? PIC_PUSH_MIN_BLOCKS_3D
     SJ = SmemJ{ji, W0, W0 * W1, ws};
   const int lane = threadIdx.x & 31;
 
-  float* ring = reinterpret_cast<float*>(queue + kQueueCap);  // TMA only
+  float* ring = reinterpret_cast<float*>(queue + P.t.queue);  // TMA only
   // The particles of this block, a contiguous share [a, b) of each species' tile
   // bucket; shares differ by at most one particle.  (By every thread: bounds
   // read from shared memory cost the 2D kernels 108 bytes of spills.)
@@ -837,7 +837,7 @@ __global__ void __launch_bounds__(kPushThreads, D == 3 ? PIC_PUSH_MIN_BLOCKS_3D
                       : one_particle<D, MODE, 0, FW0, FW1, FW2>(P, S, p, cur, sm, SJ, GA, w0, qs);
       if (kDrain && st == kStray) {
         const int slot = atomicAdd(&q_n, 1);
-        if (slot < kQueueCap) {
+        if (slot < P.t.queue) {
           queue[slot] = p;
         } else {  // full queue: this lane runs the stray through global memory now
           if (one_particle<D, MODE, 1, FW0, FW1, FW2>(P, S, p, cur, sm, SJ, GA, w0, 0.f) ==
@@ -869,14 +869,14 @@ __global__ void __launch_bounds__(kPushThreads, D == 3 ? PIC_PUSH_MIN_BLOCKS_3D
         const int qn = q_n;  // read by every thread before anyone can queue again
         if (MODE != 1) spill();
         __syncthreads();
-        if (kDrain && qn > kQueueCap / 2) drain(S, qn < kQueueCap ? qn : kQueueCap);
+        if (kDrain && qn > P.t.queue / 2) drain(S, qn < P.t.queue ? qn : P.t.queue);
       }
     }
     if (kDrain) {  // end of species: everything queued for it is processed before the next
       __syncthreads();
       const int qn = q_n;
       __syncthreads();
-      if (qn > 0) drain(S, qn < kQueueCap ? qn : kQueueCap);
+      if (qn > 0) drain(S, qn < P.t.queue ? qn : P.t.queue);
     }
   }
 
@@ -939,13 +939,13 @@ long long window_landing_floats(int dim, const TileDev& t) {
   return (long long)(particle_smem_bytes(dim, t) / sizeof(float)) - field_words(nf, t.wcells) - 31;
 }
 
-size_t particle_smem_bytes(int dim, const TileDev& t, int queue) {
+size_t particle_smem_bytes(int dim, const TileDev& t) {
   const int nf = dim == 1 ? field_floats<1>() : dim == 2 ? field_floats<2>() : field_floats<3>();
   const int jw = (dim == 2 && kJ64<2>) ? 6 : 3;  // int window words per cell
   const int jf = dim == 3 && kFoldGlobal<3> ? 0 : 3;  // float window words per cell
   // 1D/2D: the stray queue and the ring of streamed particle records
   const size_t ring = PIC_TMA_RECORDS ? (size_t)kRecStages * (1 + dim + 3) * kPushThreads : 0;
-  size_t words = (size_t)(jw + jf) * t.wstride + (dim < 3 ? queue + ring : 0);
+  size_t words = (size_t)(jw + jf) * t.wstride + (dim < 3 ? t.queue + ring : 0);
   // 2D: the same area first takes the window's tensor copy, E and B over a box
   // whose x extent is the window's widened to 16-byte ends, after up to 31
   // floats of padding to a 128-byte boundary
