@@ -205,10 +205,12 @@ int device_sms() {
 // Blocks of the particle kernel that an SM holds: the registers are for
 // PIC_PUSH_MIN_BLOCKS, shared memory may be for fewer (of 228 KB; 1 KB a block is
 // the system's, and some 200 bytes are the kernel's static ones).
+int resident_by_registers(int dim) {
+  return dim == 3 ? PIC_PUSH_MIN_BLOCKS_3D : PIC_PUSH_MIN_BLOCKS;
+}
 int resident_blocks(int dim, const TileDev& t) {
-  const int by_regs = dim == 3 ? PIC_PUSH_MIN_BLOCKS_3D : PIC_PUSH_MIN_BLOCKS;
   const int by_smem = (int)(228 * 1024 / (particle_smem_bytes(dim, t) + 1024 + 256));
-  return std::max(1, std::min(by_regs, by_smem));
+  return std::max(1, std::min(resident_by_registers(dim), by_smem));
 }
 
 // Blocks per tile for a box whose particle launch fits the GPU at once: the
@@ -217,17 +219,20 @@ int resident_blocks(int dim, const TileDev& t) {
 // work, is k (f + n / s) / e(k): k blocks on the fullest SM, n particles per
 // tile, f the fixed cost of a block (window staging, folds) and e(k) the
 // throughput of an SM with k blocks (from sweeps of s on boxes of 16 to 576
-// tiles).  0 where no s fits, where blocks would be shorter than 512 particles,
-// which the estimate does not cover, and where the best s leaves a sixth of
-// the k blocks per SM away, which is slower than more blocks than fit (3D,
-// 40^3: 58.9 us with 500 blocks, 55.7 with 750).  Measured, particle launch, against 4
-// blocks per SM rounded up: 160^2 box (100 tiles) 28.1 -> 26.0 us with 6, 256^2
-// 54.4 -> 50.9 with 2, 384^2 92.9 -> 89.4 with 1; 3D 32^3 43.5 -> 39.1 with 3,
-// 64 x 48 x 48 101.9 -> 96.6 with 1.
-long long even_splits(int dim, long long ntiles, long long per_tile, long long most) {
+// tiles).  An SM holds `resident` blocks.  0 where no s fits, where blocks would
+// be shorter than 512 particles, which the estimate does not cover, and where
+// the best s leaves a sixth of the k blocks per SM away, which is slower than
+// more blocks than fit (3D, 40^3: 58.9 us with 500 blocks, 55.7 with 750).
+// Measured, particle launch, against 4 blocks per SM rounded up: 160^2 box (100
+// tiles) 28.1 -> 26.0 us with 6, 256^2 54.4 -> 50.9 with 2, 384^2 92.9 -> 89.4
+// with 1; 3D 32^3 43.5 -> 39.1 with 3, 64 x 48 x 48 101.9 -> 96.6 with 1.  With
+// large windows, against five blocks taken to fit: 384^2 in tiles of 32^2 68 ->
+// 62, of 48^2 118 -> 106; 1D 16,000 in tiles of 1000 42 -> 33; 3D 48 x 48 x 32 in
+// tiles of 16 x 8 x 4 72 -> 54.
+long long even_splits(int dim, long long ntiles, long long per_tile, long long most, int resident) {
   const double fixed = dim == 1 ? 500.0 : dim == 2 ? 1000.0 : 1200.0;
   const double e2[4] = {0.35, 0.65, 0.85, 1.0}, e3[4] = {0.5, 0.8, 0.95, 1.0};
-  const long long sms = device_sms(), room = sms * (dim == 3 ? PIC_PUSH_MIN_BLOCKS_3D : PIC_PUSH_MIN_BLOCKS);
+  const long long sms = device_sms(), room = sms * resident;
   long long best = 0;
   double cost = 0.0;
   for (long long s = 1; s <= most && ntiles * s <= room; ++s) {
@@ -301,7 +306,20 @@ std::string derive_tiles(const pic_grid& grid, const pic_tuning& tun, long long 
   const long long fine = (per_tile + 255) / 256;
   if (sp < fill) {
     sp = fill < fine ? fill : fine;
-    const long long even = even_splits(grid.dim, ntiles, per_tile, fine);
+    // A large window leaves room for fewer blocks.  As many as the registers
+    // allow, some of them waiting for a place, where those that fit at once do not
+    // fill the SMs (3D, 48 x 48 x 32 in tiles of 10^3: 115 us a launch with 600
+    // blocks, 122 with 700), and where the tiles are very uneven, more than 3/7
+    // of their cells outside the box, which more blocks smooth out (32^3 in tiles
+    // of 10^3, 49 % outside: 73 us with 448 blocks, 81 with 128; but 130^2 in tiles
+    // of 57 x 55, 40 % outside: 74 with 603, 53 with 144).
+    long long full = ntiles, cells = 1;
+    for (int d = 0; d < grid.dim; ++d) full *= r.T[d], cells *= extent(grid, d);
+    long long even = 0;
+    if (4 * full <= 7 * cells)
+      even = even_splits(grid.dim, ntiles, per_tile, fine, resident_blocks(grid.dim, r));
+    if (even == 0)
+      even = even_splits(grid.dim, ntiles, per_tile, fine, resident_by_registers(grid.dim));
     if (even > 0) sp = even;
   }
   *t = r;
