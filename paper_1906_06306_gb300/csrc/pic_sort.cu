@@ -275,13 +275,12 @@ __device__ __forceinline__ bool two_bins(int key, bool active) {
 // warp's equal bins first took 202 us); a particle whose table slot another
 // bin holds reserves its place in the global cursor by itself.  Lanes of one
 // bin take their places one after the other, which costs most in an array that
-// is in order already.  A warp whose first and last 256th of the chunk show one
-// (no more than two bins each) therefore adds 32 at once where a round's
-// particles are of one bin.  pic_sort on an array in order, two species of
-// 16.8 M: 3D 975 -> 890 us, 2D 731 -> 688; on one in cell order, 2D 883 -> 770;
-// drifted arrays and sorts in a run within 0.3 % (with the look in every round
-// instead, 5 to 10 % more).  Scattered lane by lane, as few particles are below,
-// an array in order takes 800 and 706, a drifted one twice as long as here.
+// is in order already.  A warp whose first particles of the chunk are of no more
+// than two bins therefore adds 32 at once where a round's particles are of one.
+// pic_sort on an array in order, two species of 16.8 M: 3D 975 -> 886 us, 2D 731
+// -> 684; on one in cell order, 2D 883 -> 764; drifted arrays and sorts in a run
+// within 0.3 %.  Scattered lane by lane, as few particles are below, an array in
+// order takes 800 and 706, a drifted one twice as long as here.
 template <int D, int U>
 __global__ void __launch_bounds__(256) k_tile_scatter(const SortParams P, const SortSet Q) {
   grid_dependency();
@@ -325,9 +324,8 @@ __global__ void __launch_bounds__(256) k_tile_scatter(const SortParams P, const 
     lone_dst[r] = 0;
   }
   __syncthreads();
-  const bool in0 = t < here, in1 = (U - 1) * 256 + t < here;
-  if (two_bins(in0 ? tile_key<D>(P, c[0]) : -1, in0) &&
-      two_bins(in1 ? tile_key<D>(P, c[U - 1]) : -1, in1)) {
+  const bool in0 = t < here;
+  if (two_bins(in0 ? tile_key<D>(P, c[0]) : -1, in0)) {
     unsigned together = 0;  // bit r: round r's particles of this warp are of one bin
 #pragma unroll
     for (int r = 0; r < U; ++r) {
