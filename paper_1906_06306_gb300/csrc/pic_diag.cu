@@ -183,9 +183,10 @@ __device__ __forceinline__ void gamma_minus_1(float2 a, float2 b, float2 c, floa
 
 // Sum of m c^2 (gamma - 1).  With square root and quotient in FP64 the FP64
 // pipe bounded it, 769 us for 16.8 M particles; with terms of three floats,
-// two particles to an instruction, it takes 81 us, bound by FP32 arithmetic
+// two particles to an instruction, it takes 75 us, bound by FP32 arithmetic
 // (some 115 packed operations a pair; the reads alone would take 30 us; terms of
-// two floats, good to 2^-44 only, took 60).
+// two floats, good to 2^-44 only, took 60).  16 blocks per SM, not the 4 of the
+// other sums (81 us): with this much work in a thread, late blocks even out.
 __global__ void __launch_bounds__(256) k_kinetic(const float* __restrict__ u, long long n,
                                                  long long ld, double mc2, double* acc) {
   __shared__ double sh[32];
@@ -468,7 +469,7 @@ cudaError_t launch_field_energy(const GridDev& g, const float* F, double* acc, c
 cudaError_t launch_kinetic(const float* u, long long n, long long ld, double mc2, double* acc,
                            cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  k_kinetic<<<blocks_for_sum(n), 256, 0, st>>>(u, n, ld, mc2, acc);
+  k_kinetic<<<blocks_for(n), 256, 0, st>>>(u, n, ld, mc2, acc);
   return cudaGetLastError();
 }
 
