@@ -336,8 +336,9 @@ pic_status pic_particle_counts(pic_ctx* ctx, int64_t* n, int nout);
  * out[2+s] = sum m c^2 (gamma - 1) of species s, out[2+ns] = max |div E -
  * F^p(rho)|, out[3+ns] = rms of the same over the nodes, where rho is the
  * first-order charge on the nodes and F^p the filter_passes-fold Binomial2
- * filter (Appendix B: this residual is conserved).  Sums are accumulated in
- * double precision on the GPU.  nout must be >= 4 + nspecies. */
+ * filter (Appendix B: this residual is conserved).  Terms and sums are held to
+ * at least double precision on the GPU (FP64, sums of three floats, integers
+ * wide enough for every bit).  nout must be >= 4 + nspecies. */
 pic_status pic_energies(pic_ctx* ctx, double* out, int nout);
 
 /* Synchronise the stream and read the device status word: PIC_ERR_TIMEOUT if

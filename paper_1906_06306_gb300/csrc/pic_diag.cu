@@ -1,4 +1,4 @@
-// Diagnostics of the PIC state, accumulated in double precision on the GPU:
+// Diagnostics of the PIC state, held to at least double precision on the GPU:
 // field and kinetic energies, the first-order charge on the nodes and the
 // discrete Gauss residual div E - rho of Appendix B (arXiv:1906.06306).
 #include "pic_kernels.h"
