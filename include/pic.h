@@ -61,8 +61,9 @@ typedef enum {
 #define PIC_MAX_SPECIES 4
 
 /* Periodic box: dim = 1, 2 or 3 gridded dimensions; extents of non-gridded
- * dimensions must be 1.  nx*ny*nz must fit in int32, ny <= 65535 and
- * nz <= 21845 (launch-grid limits of the filter). */
+ * dimensions must be 1.  nx*ny*nz must fit in int32, nx with the tile window's
+ * width and 1024 points as well, ny <= 65535 and nz <= 21845 (launch-grid
+ * limits of the filter). */
 typedef struct {
   int dim;
   int nx, ny, nz;

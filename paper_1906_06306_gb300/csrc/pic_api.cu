@@ -264,6 +264,10 @@ std::string derive_tiles(const pic_grid& grid, const pic_tuning& tun, long long 
       r.T[d] = tun.tile[d] < n ? tun.tile[d] : n;
       r.nt[d] = (n + r.T[d] - 1) / r.T[d];
       r.W[d] = r.T[d] + 2 * r.H + 1;
+      // a window's and a launch grid's coordinates run past the extent, as ints:
+      // by a window's width, and by up to 1024 points of a field kernel's block
+      if ((long long)n + r.W[d] + 1024 > 0x7fffffffLL)
+        return "an extent, the tile window and 1024 points must fit in int32";
       const int ks = grid.dim == 3 ? kSubTile3[d] : grid.dim == 2 ? kSubTile2[d] : 0;
       const int sub = ks > 0 && ks < r.T[d] ? ks : r.T[d];
       r.S[d] = sub;
